@@ -130,7 +130,7 @@ int dev_smem_optin() {
 
 // Start row of level l of system s inside the batch, its blocks, E/F/W.
 void build_batch_level(gemslr_batch_ctx *B, int l, bool last, int rows_cta, BLevelHost &out) {
-    ChunkHost<float> ch;
+    ChunkHost ch;
     std::vector<int64_t> blk_r0, blk_f0, F_rp{0}, E_rp{0}, seg_r0, seg_len, seg_e0, seg_w0, seg_h0;
     std::vector<int32_t> blk_nr, blk_sys, F_ci, E_ci, seg_k, cta_seg, seg_cta0{0};
     std::vector<int64_t> cta_i0;
@@ -141,8 +141,8 @@ void build_batch_level(gemslr_batch_ctx *B, int l, bool last, int rows_cta, BLev
         const Hierarchy &h = B->sys[s];
         const HostLevel &hl = last ? h.last : h.lev[l];
         const int64_t bs = B->base[s];
-        ChunkHost<float> cs;
-        build_chunks<float>(hl.L, hl.U, hl.bp, cs, kBatchChunkRows, 1, kStageBytes);
+        ChunkHost cs;
+        build_chunks(hl.L, hl.U, hl.bp, cs, kBatchChunkRows);
         // append chunk data with offsets shifted
         const int64_t doff = (int64_t)ch.data.size();
         const int64_t coff = (int64_t)ch.off.size() - 1;

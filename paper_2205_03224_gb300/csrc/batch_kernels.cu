@@ -44,7 +44,7 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
     constexpr int kSplit = R8 / RPC;
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char *ring = smem;
-    constexpr int CPG = 1, kSlots = kRingData / kStageBytes;   // the warps share every chunk: one per copy
+    constexpr int kSlots = kMaxSlots;
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kRingData);
     uint64_t *empty = full + kSlots;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(empty + kSlots + 1);
@@ -60,14 +60,14 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kSlots; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], CPG * kBatchWarps);
+            mbar_init(&empty[s], kBatchWarps);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     if (warp == kBatchWarps) {
-        produce_chunks<CPG>(lv.C.data, lv.C.off, c0, c1, ring, full, empty, abort_flag, lv.err, lane);
+        produce_chunks(lv.C.data, lv.C.off, c0, c1, ring, full, empty, abort_flag, lv.err, lane);
         return;
     }
     const int ct = threadIdx.x;
@@ -90,10 +90,9 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
     batch_consumer_barrier();
     bool aborted = false;
     const int rr = lane / RPC, r = lane % RPC;
-    const unsigned char *base = nullptr;
     for (int c = c0; c < c1; ++c) {
         const int k = c - c0;
-        base = aborted ? nullptr : next_chunk<float, CPG>(ring, full, abort_flag, k, base);
+        const unsigned char *base = aborted ? nullptr : wait_chunk(ring, full, abort_flag, k);
         if (!aborted && !base) {
             aborted = true;
             *abort_flag = 1;
@@ -125,7 +124,7 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
                 xs[row * RPC + r] = fmaf(self, d, a0 + a1);
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[chunk_slot<CPG>(k)]);
+            if (lane == 0) mbar_arrive(&empty[k % kSlots]);
         }
         batch_consumer_barrier();
     }

@@ -174,86 +174,88 @@ template <> zc stored_entry<zc>(const Csr &T, int64_t p, int64_t pdiag) {
 
 }  // namespace
 
-template <typename VT>
-int64_t chunk_slots(int64_t maxlen) {
-    return LanesPerRow<VT>::value == 1 ? maxlen : 4 * ((maxlen + 3) / 4);
+namespace {
+
+// Rows [r0, r1) of one triangular factor in wavefront order: row ids, longest
+// first inside a wavefront (equal lengths in order), the wavefronts' ranges,
+// and every row's entries off the diagonal.
+struct Waves {
+    std::vector<int64_t> rows, ptr;
+    std::vector<int32_t> len;          // by block-local row
+};
+
+Waves order_rows(const Csr &T, int64_t r0, int64_t r1, bool upper) {
+    const std::vector<int32_t> lev = upper ? wavefronts_upper(T, r0, r1) : wavefronts_lower(T, r0, r1);
+    Waves w;
+    int32_t nw = 0;
+    for (int32_t x : lev) nw = std::max(nw, x + 1);
+    w.ptr.assign(nw + 1, 0);
+    for (int32_t x : lev) ++w.ptr[x + 1];
+    for (int32_t q = 0; q < nw; ++q) w.ptr[q + 1] += w.ptr[q];
+    w.rows.resize(r1 - r0);
+    w.len.resize(r1 - r0);
+    std::vector<int64_t> at(w.ptr.begin(), w.ptr.end() - 1);
+    for (int64_t i = r0; i < r1; ++i) {
+        int32_t c = 0;
+        for (int64_t p = T.rp[i]; p < T.rp[i + 1]; ++p) c += (T.ci[p] != i);
+        w.len[i - r0] = c;
+        w.rows[at[lev[i - r0]]++] = i;
+    }
+    for (int32_t q = 0; q < nw; ++q)
+        std::stable_sort(w.rows.begin() + w.ptr[q], w.rows.begin() + w.ptr[q + 1],
+                         [&](int64_t x, int64_t y) { return w.len[x - r0] > w.len[y - r0]; });
+    return w;
 }
 
-template <typename VT>
+int64_t diagonal(const Csr &T, int64_t i) {
+    int64_t pd = -1;
+    for (int64_t p = T.rp[i]; p < T.rp[i + 1]; ++p)
+        if (T.ci[p] == i) pd = p;
+    return pd;
+}
+
 size_t chunk_bytes(int64_t nrows, int64_t maxlen, bool upper) {
-    const size_t pr = (size_t)((nrows + 3) & ~int64_t(3));
-    const size_t ne = (size_t)(chunk_slots<VT>(maxlen) * nrows);
-    return 16 + 8 * pr + pad16(ne * 4) + pad16(ne * sizeof(VT)) + (upper ? pad16((size_t)nrows * sizeof(VT)) : 0);
+    const size_t pr = (size_t)((nrows + 3) & ~int64_t(3)), ne = (size_t)(maxlen * nrows);
+    return 16 + 8 * pr + 2 * pad16(ne * 4) + (upper ? pad16((size_t)nrows * 4) : 0);
 }
 
 // Append the chunks of one triangular factor of block [r0, r1) (see kernels.cuh).
-template <typename VT>
-void append_factor_chunks(const Csr &T, int64_t r0, int64_t r1, bool upper, ChunkHost<VT> &out, int &maxwf,
-                          int max_rows, int stage_bytes) {
-    std::vector<int32_t> lev = upper ? wavefronts_upper(T, r0, r1) : wavefronts_lower(T, r0, r1);
-    int nw = 0;
-    for (int32_t x : lev) nw = std::max(nw, x + 1);
-    maxwf = std::max(maxwf, nw);
-    std::vector<std::vector<int64_t>> rows(nw);
-    for (int64_t i = r0; i < r1; ++i) rows[lev[i - r0]].push_back(i);
-    std::vector<int64_t> nlen(r1 - r0);
-    for (int64_t i = r0; i < r1; ++i) {
-        int64_t c = 0;
-        for (int64_t p = T.rp[i]; p < T.rp[i + 1]; ++p) c += (T.ci[p] != i);
-        nlen[i - r0] = c;
-    }
-    for (int w = 0; w < nw; ++w) {
-        std::vector<int64_t> &R = rows[w];
-        std::stable_sort(R.begin(), R.end(), [&](int64_t a, int64_t c) { return nlen[a - r0] > nlen[c - r0]; });
-        if (!upper && nlen[R[0] - r0] == 0) continue;          // rows without L entries: x_i unchanged
-        size_t start = 0;
-        while (start < R.size()) {
-            const int64_t maxlen = nlen[R[start] - r0];
+void append_factor_chunks(const Csr &T, int64_t r0, int64_t r1, bool upper, ChunkHost &out, int max_rows) {
+    const Waves W = order_rows(T, r0, r1, upper);
+    for (size_t w = 0; w + 1 < W.ptr.size(); ++w) {
+        const int64_t *R = W.rows.data() + W.ptr[w];
+        const int64_t nR = W.ptr[w + 1] - W.ptr[w];
+        if (!upper && W.len[R[0] - r0] == 0) continue;          // rows without L entries: x_i unchanged
+        int64_t start = 0;
+        while (start < nR) {
+            const int64_t S = W.len[R[start] - r0];
             int64_t n = 0;
-            while (start + n < R.size() && n < max_rows &&
-                   chunk_bytes<VT>(n + 1, maxlen, upper) <= (size_t)stage_bytes)
-                ++n;
+            while (start + n < nR && n < max_rows && chunk_bytes(n + 1, S, upper) <= (size_t)kStageBytes) ++n;
             if (n == 0) fail(GEMSLR_ERR_UNSUPPORTED, "a factor row has too many entries for the staged substitution");
-            const size_t bytes = chunk_bytes<VT>(n, maxlen, upper);
-            const int64_t S = chunk_slots<VT>(maxlen);
-            out.max_slots = std::max(out.max_slots, (int)S);
+            const size_t bytes = chunk_bytes(n, S, upper);
             const size_t base = out.data.size();
             out.data.resize(base + bytes, 0);
-            unsigned char *p = out.data.data() + base;
-            int32_t *hdr = reinterpret_cast<int32_t *>(p);
+            int32_t *hdr = reinterpret_cast<int32_t *>(out.data.data() + base);
             hdr[0] = (int32_t)n;
             hdr[1] = (int32_t)S;
             hdr[2] = upper ? 1 : 0;
-            hdr[3] = 0;                                          // slices that follow in the chunk
             const int64_t pr = (n + 3) & ~int64_t(3);
             int32_t *rr = hdr + 4, *ll = rr + pr, *cc = ll + pr;
-            VT *vv = reinterpret_cast<VT *>(reinterpret_cast<unsigned char *>(cc) + pad16((size_t)(S * n) * 4));
-            VT *dd = reinterpret_cast<VT *>(reinterpret_cast<unsigned char *>(vv) + pad16((size_t)(S * n) * sizeof(VT)));
-            // the chunks store -t_ij (L) and -u_ij / u_ii (U), so that a row is
-            // x_i (times 1/u_ii) plus one sum of products (see kernels.cuh)
+            float *vv = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(cc) + pad16((size_t)(S * n) * 4));
+            float *dd = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(vv) + pad16((size_t)(S * n) * 4));
             for (int64_t t = 0; t < n; ++t) {
                 const int64_t i = R[start + t];
                 rr[t] = (int32_t)(i - r0);
-                ll[t] = (int32_t)nlen[i - r0];
-                int64_t pdiag = -1;
-                if (upper)
-                    for (int64_t pp = T.rp[i]; pp < T.rp[i + 1]; ++pp)
-                        if (T.ci[pp] == i) pdiag = pp;
-                if (upper) dd[t] = inv_entry<VT>(T, pdiag);
+                ll[t] = W.len[i - r0];
+                const int64_t pdiag = upper ? diagonal(T, i) : -1;
+                if (upper) dd[t] = inv_entry<float>(T, pdiag);
                 int64_t q = 0;
                 for (int64_t pp = T.rp[i]; pp < T.rp[i + 1]; ++pp) {
                     if (T.ci[pp] == i) continue;
-                    const int64_t e = LanesPerRow<VT>::value == 1 ? q * n + t : ((q >> 2) * n + t) * 4 + (q & 3);
-                    cc[e] = (int32_t)(T.ci[pp] - r0);
-                    vv[e] = stored_entry<VT>(T, pp, pdiag);
+                    cc[q * n + t] = (int32_t)(T.ci[pp] - r0);
+                    vv[q * n + t] = stored_entry<float>(T, pp, pdiag);
                     ++q;
                 }
-            }
-            {   // the kernels find a chunk in its group from the sizes of the chunks before it
-                const size_t pr4 = (size_t)((hdr[0] + 3) & ~3), ne4 = (size_t)hdr[1] * (size_t)hdr[0];
-                const size_t dev = 16 + 8 * pr4 + pad16(ne4 * 4) + pad16(ne4 * sizeof(VT)) +
-                                   (hdr[2] ? pad16((size_t)hdr[0] * sizeof(VT)) : 0);
-                if (dev != bytes) fail(GEMSLR_ERR_ARG, "chunk header does not describe its size");
             }
             out.off.push_back((int64_t)out.data.size());
             start += n;
@@ -261,44 +263,317 @@ void append_factor_chunks(const Csr &T, int64_t r0, int64_t r1, bool upper, Chun
     }
 }
 
+// ---- factor stream (layout in kernels.cuh) ---------------------------------------------
+// A row with more entries than this is refused (the bound of a 4 KB stage for
+// FP64 values, of 8 KB for FP32 and complex ones).
 template <typename VT>
-void build_chunks(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, ChunkHost<VT> &out, int max_rows,
-                  int max_slices, int stage_bytes) {
-    if (max_slices < 1 || max_slices > kMaxSlices) fail(GEMSLR_ERR_ARG, "slices per chunk out of range");
+bool row_too_long(int64_t len, bool upper) {
+    const int64_t slots = OneLaneRows<VT>::value ? len : 4 * ((len + 3) / 4);
+    const size_t limit = sizeof(VT) == 8 ? 4096 : 8192;
+    return 16 + 32 + pad16((size_t)slots * 4) + pad16((size_t)slots * sizeof(VT)) + (upper ? pad16(sizeof(VT)) : 0) >
+           limit;
+}
+
+// A zeroed item of `bytes` bytes, appended; returns its offset in out.data.
+size_t add_item(StreamHost &out, size_t bytes) {
+    const size_t at = out.data.size();
+    bytes = pad16(bytes);
+    if (bytes > (size_t)kMaxItemBytes) fail(GEMSLR_ERR_ARG, "factor stream item too large");
+    out.data.resize(at + bytes, 0);
+    out.off.push_back((int64_t)out.data.size());
+    out.slot_bytes = std::max(out.slot_bytes, (int)bytes);
+    return at;
+}
+
+// Slices of one factor in wavefront order, longest rows first, of at most max_rows rows.
+struct SliceRows {
+    const int64_t *rows;
+    int64_t n, longest;
+    bool sync;                         // ends its wavefront
+};
+
+template <typename VT>
+std::vector<SliceRows> cut_slices(const Waves &W, int64_t r0, bool upper, int64_t max_rows) {
+    std::vector<SliceRows> out;
+    for (size_t q = 0; q + 1 < W.ptr.size(); ++q) {
+        const int64_t *R = W.rows.data() + W.ptr[q];
+        int64_t nR = W.ptr[q + 1] - W.ptr[q];
+        // rows with nothing off the diagonal: x_i unchanged (L), or only multiplied
+        // by 1/u_ii (U: by the scaling items, in FP32 by the row itself)
+        if (!(OneLaneRows<VT>::value && upper))
+            while (nR > 0 && W.len[R[nR - 1] - r0] == 0) --nR;
+        for (int64_t at = 0; at < nR; at += max_rows) {
+            const int64_t longest = W.len[R[at] - r0];
+            if (row_too_long<VT>(longest, upper))
+                fail(GEMSLR_ERR_UNSUPPORTED, "a factor row has too many entries for the staged substitution");
+            out.push_back({R + at, std::min(max_rows, nR - at), longest, at + max_rows >= nR});
+        }
+    }
+    return out;
+}
+
+struct EntryF32 { int32_t col; float v; };
+
+// FP32 row i into its record of np pairs: pair p at slot(p), entries from 16 on to rest[(e - 16) * step].
+template <typename Slot>
+void put_row_f32(const Csr &T, int64_t r0, int64_t i, bool upper, EntryF32 *rec, Slot slot, EntryF32 *rest, int64_t step) {
+    const int64_t pdiag = upper ? diagonal(T, i) : -1;
+    int64_t e = 0;
+    for (int64_t p = T.rp[i]; p < T.rp[i + 1]; ++p) {
+        if (T.ci[p] == i) continue;
+        const EntryF32 en{(int32_t)((T.ci[p] - r0) * 4), stored_entry<float>(T, p, pdiag)};
+        if (e < 16) rec[2 * slot(e / 2) + e % 2] = en;
+        else rest[(e - 16) * step] = en;
+        ++e;
+    }
+}
+EntryF32 row_head_f32(const Csr &T, int64_t r0, int64_t i, bool upper) {
+    return {(int32_t)((i - r0) * 4), upper ? inv_entry<float>(T, diagonal(T, i)) : 1.f};
+}
+
+// FP32: rows to their heads and records; entries from 16 on to rest.
+void put_rows_f32(const Csr &T, int64_t r0, const Waves &W, bool upper, const int64_t *rows, int64_t n, int np,
+                  unsigned char *p) {
+    EntryF32 *head = reinterpret_cast<EntryF32 *>(p);
+    unsigned char *recs = p + pad16((size_t)(8 * n));
+    const bool longer = np == kLongRows;
+    const int pairs = longer ? 8 : np;
+    EntryF32 *rest = reinterpret_cast<EntryF32 *>(recs + row_bytes(pairs) * n);
+    for (int64_t t = 0; t < n; ++t) {
+        const int64_t i = rows[t], shift = longer ? 0 : pairs - (W.len[i - r0] + 1) / 2;
+        head[t] = row_head_f32(T, r0, i, upper);
+        put_row_f32(T, r0, i, upper, reinterpret_cast<EntryF32 *>(recs + row_bytes(pairs) * t),
+                    [&](int64_t pr) { return upper && !longer ? pairs - 1 - pr : pr + shift; }, rest + t, n);
+    }
+}
+
+// FP32, rows of at most 16 entries: groups of four slices.
+void append_groups(const Csr &T, int64_t r0, const Waves &W, bool upper, StreamHost &out) {
+    const int np = out.np;
+    const std::vector<SliceRows> sl = cut_slices<float>(W, r0, upper, np == 8 ? 24 : 32);   // four fit kMaxItemBytes
+    // the sequence of slices; -1: without rows (see kernels.cuh)
+    std::vector<int64_t> seq;
+    std::vector<int32_t> slice_of(W.len.size(), -1);
+    for (size_t k = 0; k < sl.size(); ++k) {
+        int64_t late = 0;
+        for (int64_t t = 0; k > 0 && t < sl[k].n; ++t) {
+            const int64_t i = sl[k].rows[t], len = W.len[i - r0];
+            int64_t e = 0;
+            for (int64_t p = T.rp[i]; p < T.rp[i + 1]; ++p) {
+                if (T.ci[p] == i) continue;
+                if (slice_of[T.ci[p] - r0] == (int32_t)k - 1)
+                    late = std::max(late, upper ? e / 2 + 1 : (len + 1) / 2 - e / 2);
+                ++e;
+            }
+        }
+        for (int64_t t = 0; t < sl[k].n; ++t) slice_of[sl[k].rows[t] - r0] = (int32_t)k;
+        if (late > kLatePairs || (upper && k == 0)) seq.push_back(-1);
+        seq.push_back((int64_t)k);
+    }
+    while (seq.size() % 4) seq.push_back(-1);
+    auto rows = [&](int64_t k) { return k < 0 ? 1 : sl[k].n; };
+    for (size_t g = 0; g < seq.size(); g += 4) {
+        size_t total = kItemHeader;
+        for (size_t q = g; q < g + 4; ++q) total += pad16((size_t)(8 * rows(seq[q]))) + (size_t)(row_bytes(np) * rows(seq[q]));
+        const size_t item = add_item(out, total);
+        unsigned char *p = out.data.data() + item;
+        size_t off = kItemHeader;
+        for (size_t q = g; q < g + 4; ++q) {
+            const int64_t k = seq[q], n = rows(k);
+            reinterpret_cast<int32_t *>(p)[q - g] = (int32_t)(off << 16) | (int32_t)(n - 1);
+            if (k < 0) *reinterpret_cast<EntryF32 *>(p + off) = {kNoRow, 1.f};
+            else put_rows_f32(T, r0, W, upper, sl[k].rows, n, np, p + off);
+            off += pad16((size_t)(8 * n)) + (size_t)(row_bytes(np) * n);
+        }
+    }
+}
+
+// FP32, any rows: one slice per item.
+void append_long_rows(const Csr &T, int64_t r0, const Waves &W, bool upper, StreamHost &out) {
+    auto bytes = [&](int64_t n, int64_t z) {
+        return kItemHeader + pad16((size_t)(8 * n)) + (size_t)((row_bytes(8) + 8 * z) * n);
+    };
+    for (const SliceRows &s : cut_slices<float>(W, r0, upper, 32)) {
+        const int64_t z = std::max<int64_t>(0, s.longest - 16);
+        for (int64_t at = 0; at < s.n;) {
+            int64_t n = 1;
+            while (at + n < s.n && bytes(n + 1, z) <= (size_t)kMaxItemBytes) ++n;
+            const size_t item = add_item(out, bytes(n, z));
+            int32_t *h = reinterpret_cast<int32_t *>(out.data.data() + item);
+            h[0] = (int32_t)n - 1;
+            h[2] = (int32_t)z;
+            unsigned char *p = out.data.data() + item + kItemHeader;
+            EntryF32 *rest = reinterpret_cast<EntryF32 *>(p + pad16((size_t)(8 * n)) + row_bytes(8) * n);
+            for (int64_t k = 0; k < z * n; ++k) rest[k] = {-1, 0.f};
+            put_rows_f32(T, r0, W, upper, s.rows + at, n, kLongRows, p);
+            at += n;
+        }
+    }
+}
+
+// FP64 and complex slices of one block, back to back, before they are packed.
+struct LaneSlices {
+    std::vector<unsigned char> data;
+    std::vector<size_t> off{0};
+    unsigned char *add(size_t bytes, int64_t n, int64_t z, int flags) {
+        const size_t at = data.size();
+        data.resize(at + pad16(bytes), 0);
+        off.push_back(data.size());
+        int32_t *h = reinterpret_cast<int32_t *>(data.data() + at);
+        h[0] = (int32_t)n - 1;
+        h[2] = (int32_t)z;
+        h[3] = flags;
+        return data.data() + at + kItemHeader;
+    }
+};
+
+template <typename VT>
+void append_lanes(const Csr &T, int64_t r0, const Waves &W, bool upper, int np, LaneSlices &out) {
+    const size_t lb = lane_bytes<VT>(np), tb = pad16(sizeof(VT) + 4);
+    auto bytes = [&](int64_t n, int64_t m) {
+        return kItemHeader + (size_t)(4 * n) * (lb + (size_t)std::max<int64_t>(0, (m + 3) / 4 - 4) * tb);
+    };
+    for (const SliceRows &s : cut_slices<VT>(W, r0, upper, 32)) {
+        for (int64_t at = 0; at < s.n;) {
+            int64_t n = 1;
+            while (at + n < s.n && bytes(n + 1, s.longest) <= (size_t)kMaxItemBytes) ++n;
+            const int cls = s.longest <= 1 ? kLane1 : s.longest <= 2 ? kLane2 : s.longest <= 4 ? kLane4 : s.longest <= 16 ? kLaneFull : kLaneLong;
+            unsigned char *p = out.add(bytes(n, s.longest), n, s.longest,
+                                       cls << kLaneShift | (s.sync && at + n == s.n ? kSync : 0));
+            for (int64_t t = 0; t < n; ++t) {
+                const int64_t i = s.rows[at + t], pdiag = upper ? diagonal(T, i) : -1;
+                auto put = [&](unsigned char *rv, unsigned char *rc, int64_t col, VT v) {
+                    *reinterpret_cast<VT *>(rv) = v;
+                    *reinterpret_cast<int32_t *>(rc) = (int32_t)((col - r0) * (int64_t)sizeof(VT));
+                };
+                for (int64_t q = 0; q < 4; ++q)
+                    *reinterpret_cast<int32_t *>(p + lb * (4 * t + q) + np * (sizeof(VT) + 4)) =
+                        (int32_t)((i - r0) * (int64_t)sizeof(VT));
+                int64_t e = 0;
+                for (int64_t pp = T.rp[i]; pp < T.rp[i + 1]; ++pp) {
+                    if (T.ci[pp] == i) continue;
+                    const int64_t k = e >> 2, lane = 4 * t + (e & 3);
+                    unsigned char *rec = p + lb * lane, *rest = p + lb * 4 * n + tb * ((k - 4) * 4 * n + lane);
+                    const VT v = stored_entry<VT>(T, pp, pdiag);
+                    if (k < 4) put(rec + k * sizeof(VT), rec + np * sizeof(VT) + 4 * k, T.ci[pp], v);
+                    else put(rest, rest + sizeof(VT), T.ci[pp], v);
+                    ++e;
+                }
+            }
+            at += n;
+        }
+    }
+}
+
+// The x_i / u_ii products of a block between L and U.
+template <typename VT>
+void append_scaling(const Csr &U, int64_t r0, int64_t nr, LaneSlices &out) {
+    const int64_t step = 4096 / (int64_t)sizeof(VT);
+    for (int64_t i0 = 0; i0 < nr; i0 += step) {
+        const int64_t n = std::min(step, nr - i0);
+        VT *d = reinterpret_cast<VT *>(out.add(kItemHeader + (size_t)n * sizeof(VT), n, i0,
+                                                  kLaneScale << kLaneShift | (i0 + n == nr ? kSync : 0)));
+        for (int64_t i = 0; i < n; ++i) d[i] = inv_entry<VT>(U, diagonal(U, r0 + i0 + i));
+    }
+}
+
+// Slices to items: consecutive rounds of one slice per consumer are joined while
+// every consumer's share keeps its class and stays within kLaneItemBytes.  Returns the slices with kSync.
+int32_t pack_lanes(LaneSlices &s, StreamHost &out) {
+    const size_t nc = out.consumers, ns = s.off.size() - 1;
+    auto header = [&](size_t k) { return reinterpret_cast<int32_t *>(s.data.data() + s.off[k]); };
+    auto bytes = [&](size_t k) { return s.off[k + 1] - s.off[k]; };
+    auto cls = [&](size_t k) { return header(k)[3] >> kLaneShift & 7; };
+    int32_t nsync = 0;
+    for (size_t k = 0; k < ns; ++k) {
+        int between = 0;                              // wavefronts that end in the other consumers' slices
+        for (size_t j = k; j-- > 0 && j + nc > k;) between += header(j)[3] & kSync ? 1 : 0;
+        nsync += header(k)[3] & kSync ? 1 : 0;
+        header(k)[3] |= between << 24;
+    }
+    for (size_t k0 = 0; k0 < ns;) {
+        std::vector<size_t> share(nc, 0);
+        size_t k1 = k0;
+        while (k1 < ns) {
+            bool fits = true;
+            for (size_t c = 0; c < nc && k1 + c < ns; ++c)
+                fits = fits && (k1 == k0 || (cls(k1 + c) == cls(k0 + c) && cls(k0 + c) != kLaneScale &&
+                                             share[c] + bytes(k1 + c) <= (size_t)kLaneItemBytes));
+            if (!fits) break;
+            for (size_t c = 0; c < nc && k1 + c < ns; ++c) share[c] += bytes(k1 + c);
+            k1 = std::min(ns, k1 + nc);
+        }
+        for (size_t c = 0; c < nc && k0 + c < k1; ++c) {
+            size_t at = add_item(out, share[c]);
+            for (size_t k = k0 + c; k < k1; k += nc) {
+                header(k)[1] = k + nc < k1 ? (int32_t)bytes(k) : 0;
+                std::memcpy(out.data.data() + at, s.data.data() + s.off[k], bytes(k));
+                at += bytes(k);
+            }
+        }
+        k0 = k1;
+    }
+    return nsync;
+}
+
+}  // namespace
+
+void build_chunks(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, ChunkHost &out, int max_rows) {
     validate_tri(L, bp, false);
     validate_tri(U, bp, true);
     for (size_t b = 0; b + 1 < bp.size(); ++b) {
-        const size_t first = out.off.size() - 1;
-        append_factor_chunks<VT>(L, bp[b], bp[b + 1], false, out, out.maxwf_L, max_rows, stage_bytes);
-        append_factor_chunks<VT>(U, bp[b], bp[b + 1], true, out, out.maxwf_U, max_rows, stage_bytes);
-        if (max_slices >= 2) {
-            // join up to max_slices consecutive slices into one chunk (<= stage_bytes)
-            // by dropping the boundaries between them; the header of every slice but
-            // the chunk's last says that another one follows
-            std::vector<int64_t> keep(out.off.begin(), out.off.begin() + (int64_t)first + 1);
-            size_t c = first;
-            const size_t last = out.off.size() - 1;
-            while (c < last) {
-                const int64_t a0 = out.off[c];
-                size_t e = c + 1;                    // slices [c, e) form the chunk
-                while (e < last && (int)(e + 1 - c) <= max_slices && out.off[e + 1] - a0 <= (int64_t)stage_bytes) ++e;
-                for (size_t t = c; t + 1 < e; ++t) reinterpret_cast<int32_t *>(out.data.data() + out.off[t])[3] = 1;
-                keep.push_back(out.off[e]);
-                c = e;
-            }
-            out.off.swap(keep);
-        }
+        append_factor_chunks(L, bp[b], bp[b + 1], false, out, max_rows);
+        append_factor_chunks(U, bp[b], bp[b + 1], true, out, max_rows);
         out.blk_chunk.push_back((int32_t)(out.off.size() - 1));
     }
     if (out.data.empty()) out.data.resize(16, 0);
 }
 
+template <typename VT>
+void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, StreamHost &out) {
+    validate_tri(L, bp, false);
+    validate_tri(U, bp, true);
+    const size_t nb = bp.size() - 1;
+    std::vector<Waves> wl(nb), wu(nb);
+    int32_t longest = 0;
+    for (size_t b = 0; b < nb; ++b) {
+        wl[b] = order_rows(L, bp[b], bp[b + 1], false);
+        wu[b] = order_rows(U, bp[b], bp[b + 1], true);
+        for (int32_t x : wl[b].len) longest = std::max(longest, x);
+        for (int32_t x : wu[b].len) longest = std::max(longest, x);
+        out.maxwf_L = std::max(out.maxwf_L, (int)wl[b].ptr.size() - 1);
+        out.maxwf_U = std::max(out.maxwf_U, (int)wu[b].ptr.size() - 1);
+    }
+    constexpr bool one = OneLaneRows<VT>::value;
+    out.np = trsv_record(one, longest);
+    int64_t nwave = 1;
+    for (size_t b = 0; b < nb; ++b) nwave += (int64_t)(wl[b].ptr.size() + wu[b].ptr.size());
+    out.consumers = !one ? trsv_sets((double)(2 * bp.back()) / (double)nwave) : out.np == kLongRows ? 1 : 4;
+    for (size_t b = 0; b < nb; ++b) {
+        const int64_t r0 = bp[b];
+        if constexpr (one) {
+            const size_t first = out.off.size();
+            auto append = out.np == kLongRows ? append_long_rows : append_groups;
+            append(L, r0, wl[b], false, out);
+            out.split.push_back((int32_t)(out.off.size() - first));
+            append(U, r0, wu[b], true, out);
+        } else {
+            LaneSlices s;
+            append_lanes<VT>(L, r0, wl[b], false, out.np, s);
+            append_scaling<VT>(U, r0, bp[b + 1] - r0, s);
+            append_lanes<VT>(U, r0, wu[b], true, out.np, s);
+            out.split.push_back(pack_lanes(s, out));
+        }
+        out.blk_item.push_back((int32_t)(out.off.size() - 1));
+        wl[b] = Waves();
+        wu[b] = Waves();
+    }
+    if (out.data.empty()) out.data.resize(16, 0);
+}
 
-template void build_chunks<float>(const Csr &, const Csr &, const std::vector<int64_t> &, ChunkHost<float> &, int, int,
-                                  int);
-template void build_chunks<double>(const Csr &, const Csr &, const std::vector<int64_t> &, ChunkHost<double> &, int,
-                                   int, int);
-template void build_chunks<zc>(const Csr &, const Csr &, const std::vector<int64_t> &, ChunkHost<zc> &, int, int, int);
+template void build_stream<float>(const Csr &, const Csr &, const std::vector<int64_t> &, StreamHost &);
+template void build_stream<double>(const Csr &, const Csr &, const std::vector<int64_t> &, StreamHost &);
+template void build_stream<zc>(const Csr &, const Csr &, const std::vector<int64_t> &, StreamHost &);
 
 namespace {
 
@@ -314,17 +589,23 @@ void upload_level(const HostLevel &hl, int64_t n, bool schur, Arena &a, DevLevel
     int64_t maxrows = 0;
     for (size_t b = 0; b + 1 < hl.bp.size(); ++b) maxrows = std::max(maxrows, hl.bp[b + 1] - hl.bp[b]);
     d.smem_rows = (kRingBytes + maxrows * (int64_t)sizeof(VT) <= smem_limit) ? (int)maxrows : 0;
-    ChunkHost<VT> ch;
-    build_chunks<VT>(hl.L, hl.U, hl.bp, ch, kChunkRows, LanesPerRow<VT>::value == 1 ? kMaxSlices : 1,
-                     StageBytesOf<VT>::value);
-    v.C.data = a.upload(ch.data);
-    v.C.off = a.upload(ch.off);
-    v.C.blk_chunk = a.upload(ch.blk_chunk);
-    v.max_slots = ch.max_slots;
-    d.nwf_L = ch.maxwf_L;
-    d.nwf_U = ch.maxwf_U;
-    d.nchunks = (int64_t)ch.off.size() - 1;
-    d.nnz_tri = hl.L.nnz() + hl.U.nnz();
+    StreamHost sh;
+    build_stream<VT>(hl.L, hl.U, hl.bp, sh);
+    v.S.data = a.upload(sh.data);
+    v.S.off = a.upload(sh.off);
+    v.S.blk_item = a.upload(sh.blk_item);
+    v.S.split = a.upload(sh.split);
+    v.S.np = sh.np;
+    v.S.consumers = sh.consumers;
+    // the ring: up to kItemDepth slots per consumer, in twice kRingData where the
+    // vector leaves that much (more bytes in flight), at least one
+    const int64_t room = (d.smem_rows ? smem_limit - (int64_t)pad16(d.smem_rows * sizeof(VT)) : (int64_t)kRingBytes) -
+                         (int64_t)sizeof(StreamHead);
+    v.S.slot_bytes = std::max(sh.slot_bytes, 128);
+    const int64_t depth = std::min<int64_t>(room, 2 * kRingData) / ((int64_t)v.S.slot_bytes * sh.consumers);
+    v.S.slots = sh.consumers * (int)std::max<int64_t>(1, std::min<int64_t>(depth, kItemDepth));
+    d.nwf_L = sh.maxwf_L;
+    d.nwf_U = sh.maxwf_U;
     if (schur) {
         std::vector<int32_t> fci(hl.F.ci.size());
         for (size_t p = 0; p < fci.size(); ++p) fci[p] = (int32_t)(hl.F.ci[p] + hl.e);

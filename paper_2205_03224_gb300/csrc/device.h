@@ -32,13 +32,17 @@ void profile_reset();
 int profile_read(char *names, size_t len, double *ms, int64_t *counts, int maxn);
 uint64_t launches_total();
 
-// ---- launchers (kernels.cu) --------------------------------------------------
+// ---- launchers (kernels.cu, trsv.cu) --------------------------------------------------
 // pl: the previous level's pending W u (MODE 0 only; default: none).
 template <typename VT, typename WT>
 void launch_trsv(const LevelView<VT, WT> &lv, int mode, int smem_rows, const IoT<VT> *in, VT *work,
                  IoT<VT> *out_final, VT *scratch, cudaStream_t st,
                  const PendingLowRank<VT, WT> &pl = PendingLowRank<VT, WT>());
 template <typename VT, typename WT> void set_trsv_smem_limit(int bytes);
+// the kernel variant of a level: StreamView::np for its longest row; sets of
+// warps (FP64) for its mean rows per wavefront
+int trsv_record(bool one_lane, int longest);
+int trsv_sets(double width);
 template <typename VT, typename WT>
 void launch_couple(const LevelView<VT, WT> &lv, const IoT<VT> *in, VT *work, VT *partial, unsigned *counter,
                    VT *u, cudaStream_t st, const PendingLowRank<VT, WT> &pl = PendingLowRank<VT, WT>());
@@ -118,21 +122,24 @@ template <typename T> inline std::vector<T> convert(const std::vector<double> &x
     return y;
 }
 
-template <typename VT>
-struct ChunkHost {
+// Factors L, U of one level in the layouts of kernels.cuh (host copies).
+struct ChunkHost {                     // batched substitutions
     std::vector<unsigned char> data;
     std::vector<int64_t> off{0};
     std::vector<int32_t> blk_chunk{0};
-    int maxwf_L = 0, maxwf_U = 0;
-    int max_slots = 0;                 // largest S of any slice
 };
+void build_chunks(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, ChunkHost &out, int max_rows);
 
-// Chunks (layout in kernels.cuh) of the block-diagonal factors L, U of one
-// level: slices of at most max_rows row slots, up to max_slices (1 ..
-// kMaxSlices) consecutive slices per chunk of at most stage_bytes.
+struct StreamHost {                    // single-system substitutions (see StreamView)
+    std::vector<unsigned char> data;
+    std::vector<int64_t> off{0};
+    std::vector<int32_t> blk_item{0}, split;
+    int np = 0, consumers = 1;
+    int slot_bytes = 0;                // largest item
+    int maxwf_L = 0, maxwf_U = 0;      // wavefronts (largest over the blocks)
+};
 template <typename VT>
-void build_chunks(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, ChunkHost<VT> &out, int max_rows,
-                  int max_slices, int stage_bytes);
+void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, StreamHost &out);
 
 // ---- device memory arena ------------------------------------------------------------
 class Arena {
@@ -166,8 +173,6 @@ struct DevLevel {
     LevelView<VT, WT> view{};
     int smem_rows = 0;          // dynamic shared memory rows of the trsv kernel (0 = global)
     int nwf_L = 0, nwf_U = 0;   // wavefront counts (max over blocks)
-    int64_t nnz_tri = 0;
-    int64_t nchunks = 0;
 };
 
 // Inner GMRES of the root level (inner.cu); k = 0: the standard application.

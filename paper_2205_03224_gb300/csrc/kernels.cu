@@ -25,260 +25,12 @@
 #include <cstdio>
 
 #include "device.h"
+#include "lowrank.cuh"
 #include "ptx.cuh"
 
 namespace gemslr {
 
 namespace {
-
-template <typename T> __device__ __forceinline__ float to_f(T v);
-template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-template <typename VT, typename WT> __device__ __forceinline__ VT wval(WT w) { return (VT)to_f(w); }
-template <> __device__ __forceinline__ double wval<double, double>(double w) { return w; }
-template <> __device__ __forceinline__ zc wval<zc, zc>(zc w) { return w; }
-// an entry of W^H (the correction is W H W^H; for real data W^T)
-template <typename VT, typename WT> __device__ __forceinline__ VT wval_h(WT w) { return wval<VT, WT>(w); }
-template <> __device__ __forceinline__ zc wval_h<zc, zc>(zc w) { return conj(w); }
-
-// Row g's share of the previous level's W u (see PendingLowRank): sixteen
-// columns at a time with all their loads issued first (columns past k load
-// the last column again and are multiplied by zero).  u is read through L2:
-// the coupling kernel that reads it also rewrites it in its finisher.
-template <typename VT, typename WT>
-__device__ __forceinline__ VT pending_row(const PendingLowRank<VT, WT> &pl, int64_t g) {
-    const WT *w = pl.W + (g - pl.row0);
-    VT a0 = 0, a1 = 0;
-    for (int c0 = 0; c0 < pl.k; c0 += 16) {
-        WT wv[16];
-        VT uv[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int c = min(c0 + q, pl.k - 1);
-            wv[q] = w[(int64_t)c * pl.ld];
-            uv[q] = c0 + q < pl.k ? ldcg(pl.u + c) : (VT)0;
-        }
-#pragma unroll
-        for (int q = 0; q < 16; q += 2) {
-            a0 += wval<VT, WT>(wv[q]) * uv[q];
-            a1 += wval<VT, WT>(wv[q + 1]) * uv[q + 1];
-        }
-    }
-    return a0 + a1;
-}
-
-
-// ---- level-scheduled substitutions over one block --------------------------
-// One CTA per diagonal block.  Warp kConsumerWarps is the producer: it
-// streams the block's chunks (see kernels.cuh) into a shared-memory ring,
-// CPG chunks per bulk copy completing on an mbarrier.  The
-// consumer warps keep the block's vector x in shared memory (or global memory
-// for blocks that do not fit) and, chunk by chunk, compute
-//   x_i = (x_i - sum_j T_ij x_j) * (U ? 1/u_ii : 1)
-// with the rows of a chunk spread over the consumer warps, lane per row.
-// MODE 0: right-hand side from `in` (FP64 user vector) or `work`; result in work.
-// MODE 1: right-hand side F y2 (gathered from work's tail); work[rows] -= result.
-template <typename VT, typename WT, int MODE, bool SMEM, int NE>
-__global__ void __launch_bounds__(kTrsvThreads2)
-k_trsv(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restrict__ work,
-       IoT<VT> *__restrict__ out_final, VT *__restrict__ scratch, const PendingLowRank<VT, WT> pl) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    unsigned char *ring = smem;
-    // FP32: kGroupChunks chunks per copy, one per consumer warp; FP64: one
-    constexpr int CPG = LanesPerRow<VT>::value == 1 ? kGroupChunks : 1;
-    constexpr int SB = StageBytesOf<VT>::value;
-    constexpr int kSlots = kRingData / (CPG * SB);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kRingData);
-    uint64_t *empty = full + kSlots;
-    uint64_t *cbar = empty + kSlots;
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(cbar + 1);
-    VT *xs_smem = reinterpret_cast<VT *>(smem + kRingBytes);
-
-    const int b = blockIdx.x;
-    const int64_t r0 = lv.blk_row[b];
-    const int nr = (int)(lv.blk_row[b + 1] - r0);
-    if (nr == 0) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c0 = lv.C.blk_chunk[b], c1 = lv.C.blk_chunk[b + 1];
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kSlots; ++s) {
-            mbar_init(&full[s], 1);
-            // FP32 chunks are released by one consumer warp, FP64 chunks by all of them
-            mbar_init(&empty[s], CPG * (LanesPerRow<VT>::value == 1 ? 1 : kConsumerWarps));
-        }
-        mbar_init(cbar, kConsumerWarps);
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-
-    if (warp == kConsumerWarps) {            // producer warp
-        produce_chunks<CPG, SB>(lv.C.data, lv.C.off, c0, c1, ring, full, empty, abort_flag, lv.err, lane);
-        return;
-    }
-
-    // consumer warps: every chunk ends with the same named barrier, so a warp
-    // whose wait expired keeps the barrier count of the others (no deadlock)
-    const int ct = threadIdx.x;                        // 0 .. 32*kConsumerWarps-1
-    constexpr int NC = 32 * kConsumerWarps;
-    VT *mine = work + lv.s + r0;
-    VT *xs = SMEM ? xs_smem : (MODE == 1 ? scratch + r0 : mine);
-    if (MODE == 1) {
-        // right-hand side F y2: zero, then the (few) block rows with F entries,
-        // one thread per row so that their index and value loads overlap
-        for (int i = ct; i < nr; i += NC) xs[i] = (VT)0;
-        consumer_barrier();
-        // four rows per thread at a time, each step's loads for all of them in
-        // flight together (row ids, row extents, the first two entries, x)
-        const int f1 = lv.F_blk[b + 1];
-        for (int t0 = lv.F_blk[b] + ct; t0 < f1; t0 += 4 * NC) {
-            int64_t g[4], pa[4], pb[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) g[u] = t0 + u * NC < f1 ? lv.F_rows[t0 + u * NC] : -1;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                pa[u] = g[u] >= 0 ? lv.F_rp[g[u]] : 0;
-                pb[u] = g[u] >= 0 ? lv.F_rp[g[u] + 1] : 0;
-            }
-            int32_t cc[4][2];
-            VT vv[4][2];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const bool live = pa[u] + q < pb[u];
-                    const int64_t pq = live ? pa[u] + q : pa[u];
-                    cc[u][q] = g[u] >= 0 ? lv.F_ci[pq] : 0;
-                    vv[u][q] = live ? lv.F_v[pq] : (VT)0;
-                }
-            VT xv[4][2];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int q = 0; q < 2; ++q) xv[u][q] = g[u] >= 0 ? work[cc[u][q]] : (VT)0;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (g[u] < 0) continue;
-                VT acc = vv[u][0] * xv[u][0] + vv[u][1] * xv[u][1];
-                for (int64_t p = pa[u] + 2; p < pb[u]; ++p) acc += lv.F_v[p] * work[lv.F_ci[p]];
-                xs[g[u] - r0] = acc;
-            }
-        }
-    } else if (pl.W) {
-        // right-hand side z2 + W u of the previous level (MODE 0, never the first level)
-        for (int i = ct; i < nr; i += NC) xs[i] = mine[i] + pending_row<VT, WT>(pl, lv.s + r0 + i);
-    } else if (in || SMEM) {
-        // eight independent loads in flight per thread
-        const IoT<VT> *src_d = in ? in + lv.s + r0 : nullptr;
-        for (int i0 = ct; i0 < nr; i0 += 8 * NC) {
-            VT v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = i0 + u * NC;
-                v[u] = i < nr ? (src_d ? (VT)src_d[i] : mine[i]) : (VT)0;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (i0 + u * NC < nr) xs[i0 + u * NC] = v[u];
-        }
-    }
-    consumer_barrier();
-    if constexpr (LanesPerRow<VT>::value == 1) {
-        // FP32: the consumer warps take the chunks in turn, one lane per row,
-        // each loading its next chunk into registers while the others work.
-        consume_chunks_round_robin<VT, NE, SB>(ring, full, empty, abort_flag, c1 - c0, xs, warp, lane);
-    } else {
-        bool aborted = false;
-        const int r = lane >> 2, sub = lane & 3;
-        const unsigned char *base = nullptr;
-        for (int c = c0; c < c1; ++c) {
-            const int k = c - c0;
-            base = aborted ? nullptr : next_chunk<VT, CPG, SB>(ring, full, abort_flag, k, base);
-            if (!aborted && !base) {
-                aborted = true;
-                *abort_flag = 1;
-            }
-            if (!aborted) {
-                const int *hdr = reinterpret_cast<const int *>(base);
-                const int nrow = hdr[0], S = hdr[1], upper = hdr[2];
-                const int pr = (nrow + 3) & ~3;
-                const int *rows = hdr + 4;
-                const int *lens = rows + pr;
-                const int *cols = lens + pr;
-                const VT *vals = reinterpret_cast<const VT *>(cols + (size_t)S * nrow);
-                const int per = (nrow + kConsumerWarps - 1) / kConsumerWarps;   // rows of this warp (<= 8)
-                if (warp * per < nrow) {                                       // idle warps skip the FP64 work
-                    // x_row = x_row d + sum_j v_j x_j with v_j = -t_row,j (d = 1, L) or
-                    // -u_row,j / u_row,row (d = 1 / u_row,row, U): the padded slots hold
-                    // column 0 and value 0, so every lane loads its first four entries
-                    // unconditionally, all loads before the arithmetic, and adds them in
-                    // two short chains (dependent FP64 operations are slow on this part);
-                    // inactive lanes read row slot 0 and their sums are discarded
-                    const int t = warp * per + r;
-                    const bool active = r < per && t < nrow;
-                    const int tt = active ? t : 0;
-                    const int kq = S >> 2;
-                    const int row = rows[tt];
-                    int cq[4];
-                    VT vq[4], xq[4];
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {                            // slots past S: column 0, value 0
-                        const int e = (kk * nrow + tt) * 4 + sub;
-                        cq[kk] = kk < kq ? cols[e] : 0;
-                        vq[kk] = kk < kq ? vals[e] : (VT)0;
-                    }
-                    VT a0 = 0;
-                    if (sub == 0) {
-                        a0 = xs[row];
-                        if (upper) a0 *= vals[(size_t)S * nrow + tt];          // dinv follows vals
-                    }
-                    VT a1 = 0;
-                    if constexpr (IsComplex<VT>::value) {
-                        // a complex product is four FP64 FMAs: skip the slots past kq
-                        // (uniform over the chunk)
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) xq[kk] = kk < kq ? xs[cq[kk]] : (VT)0;
-                        if (kq > 0) a0 += vq[0] * xq[0];
-                        if (kq > 1) a1 = vq[1] * xq[1];
-                        if (kq > 2) a0 += vq[2] * xq[2];
-                        if (kq > 3) a1 += vq[3] * xq[3];
-                    } else {
-                        // FP64: all four slots, no branches (padded slots add 0 * x_0)
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) xq[kk] = xs[cq[kk]];
-                        a1 = vq[1] * xq[1];
-                        a0 += vq[0] * xq[0];
-                        a1 += vq[3] * xq[3];
-                        a0 += vq[2] * xq[2];
-                    }
-                    for (int kk = 4; kk < kq; ++kk) {                          // rows of more than 16 entries
-                        const int e = (kk * nrow + tt) * 4 + sub;
-                        a0 += vals[e] * xs[cols[e]];
-                    }
-                    VT acc = a0 + a1;
-                    acc += shfl_xor(acc, 1);
-                    acc += shfl_xor(acc, 2);
-                    if (active && sub == 0) xs[row] = acc;
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[chunk_slot<CPG, SB>(k)]);
-            }
-            consumer_barrier();
-        }
-    }
-    consumer_barrier();
-    if (*abort_flag) {
-        if (ct == 0) atomicExch(lv.err, 1);
-        return;
-    }
-    for (int i = ct; i < nr; i += NC) {
-        VT y = xs[i];
-        if (MODE == 1) y = mine[i] - y;
-        if (SMEM || MODE == 1) mine[i] = y;
-        if (out_final) out_final[lv.s + r0 + i] = (IoT<VT>)y;
-    }
-}
 
 // z2 = b2 - E z1 on rows [row0, row1) of the tail, then partial W^T z2 (W^H z2
 // for the complex hierarchy).
@@ -1507,69 +1259,6 @@ static int grid_for(int64_t n, int threads, int cap) {
 }
 
 template <typename VT, typename WT>
-void launch_trsv(const LevelView<VT, WT> &lv, int mode, int smem_rows, const IoT<VT> *in, VT *work,
-                 IoT<VT> *out_final, VT *scratch, cudaStream_t st, const PendingLowRank<VT, WT> &pl) {
-    if (lv.nblk == 0) return;
-    const bool smem = smem_rows > 0;
-    const size_t bytes = kRingBytes + (smem ? (size_t)smem_rows * sizeof(VT) : 0);
-    // FP32: register slots sized to the level's longest row (4, 8, 12 or 16)
-    const int ne = LanesPerRow<VT>::value != 1 ? 16 : lv.max_slots <= 4 ? 4 : lv.max_slots <= 8 ? 8
-                                                 : lv.max_slots <= 12 ? 12 : 16;
-#define GEMSLR_TRSV(M, S, N) \
-    k_trsv<VT, WT, M, S, N><<<lv.nblk, kTrsvThreads2, bytes, st>>>(lv, in, work, out_final, scratch, pl)
-#define GEMSLR_TRSV_NE(M, S)                  \
-    switch (ne) {                             \
-        case 4: GEMSLR_TRSV(M, S, 4); break;  \
-        case 8: GEMSLR_TRSV(M, S, 8); break;  \
-        case 12: GEMSLR_TRSV(M, S, 12); break; \
-        default: GEMSLR_TRSV(M, S, 16); break; \
-    }
-    if constexpr (LanesPerRow<VT>::value == 1) {
-        if (mode == 0) {
-            if (smem) { GEMSLR_TRSV_NE(0, true) }
-            else { GEMSLR_TRSV_NE(0, false) }
-        } else {
-            if (smem) { GEMSLR_TRSV_NE(1, true) }
-            else { GEMSLR_TRSV_NE(1, false) }
-        }
-    } else {
-        if (mode == 0) {
-            if (smem) GEMSLR_TRSV(0, true, 16);
-            else GEMSLR_TRSV(0, false, 16);
-        } else {
-            if (smem) GEMSLR_TRSV(1, true, 16);
-            else GEMSLR_TRSV(1, false, 16);
-        }
-    }
-#undef GEMSLR_TRSV_NE
-#undef GEMSLR_TRSV
-    count_launch();
-}
-
-template <typename VT, typename WT>
-void set_trsv_smem_limit(int bytes) {
-    auto set = [&](auto fn, int b) { cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, b); };
-    set(k_trsv<VT, WT, 0, true, 16>, bytes);
-    set(k_trsv<VT, WT, 1, true, 16>, bytes);
-    set(k_trsv<VT, WT, 0, false, 16>, kRingBytes);
-    set(k_trsv<VT, WT, 1, false, 16>, kRingBytes);
-    if constexpr (LanesPerRow<VT>::value == 1) {
-        set(k_trsv<VT, WT, 0, true, 4>, bytes);
-        set(k_trsv<VT, WT, 0, true, 8>, bytes);
-        set(k_trsv<VT, WT, 0, true, 12>, bytes);
-        set(k_trsv<VT, WT, 1, true, 4>, bytes);
-        set(k_trsv<VT, WT, 1, true, 8>, bytes);
-        set(k_trsv<VT, WT, 1, true, 12>, bytes);
-        set(k_trsv<VT, WT, 0, false, 4>, kRingBytes);
-        set(k_trsv<VT, WT, 0, false, 8>, kRingBytes);
-        set(k_trsv<VT, WT, 0, false, 12>, kRingBytes);
-        set(k_trsv<VT, WT, 1, false, 4>, kRingBytes);
-        set(k_trsv<VT, WT, 1, false, 8>, kRingBytes);
-        set(k_trsv<VT, WT, 1, false, 12>, kRingBytes);
-    }
-}
-
-template <typename VT, typename WT>
 void launch_couple(const LevelView<VT, WT> &lv, const IoT<VT> *in, VT *work, VT *partial, unsigned *counter,
                    VT *u, cudaStream_t st, const PendingLowRank<VT, WT> &pl) {
     if (lv.stail == 0) return;
@@ -1578,16 +1267,6 @@ void launch_couple(const LevelView<VT, WT> &lv, const IoT<VT> *in, VT *work, VT 
 }
 
 
-template void launch_trsv<double, double>(const LevelView<double, double> &, int, int, const double *, double *,
-                                          double *, double *, cudaStream_t, const PendingLowRank<double, double> &);
-template void launch_trsv<float, __nv_bfloat16>(const LevelView<float, __nv_bfloat16> &, int, int, const double *,
-                                                float *, double *, float *, cudaStream_t,
-                                                const PendingLowRank<float, __nv_bfloat16> &);
-template void launch_trsv<zc, zc>(const LevelView<zc, zc> &, int, int, const zc *, zc *, zc *, zc *, cudaStream_t,
-                                  const PendingLowRank<zc, zc> &);
-template void set_trsv_smem_limit<double, double>(int);
-template void set_trsv_smem_limit<zc, zc>(int);
-template void set_trsv_smem_limit<float, __nv_bfloat16>(int);
 template void launch_couple<double, double>(const LevelView<double, double> &, const double *, double *, double *,
                                             unsigned *, double *, cudaStream_t,
                                             const PendingLowRank<double, double> &);

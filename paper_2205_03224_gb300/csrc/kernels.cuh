@@ -9,58 +9,100 @@
 
 namespace gemslr {
 
-constexpr int kTrsvThreads = 512;
 constexpr int kCoupleRows = 256;    // tail rows per CTA in the E / W^T kernel
 constexpr int kMaxRank = 160;       // k_eff upper bound in the correction kernels
 constexpr int kReduceThreads = 256;
 constexpr int kMaxCols = 160;     // Krylov columns per Gram-Schmidt pass (m + 1 <= kMaxCols)
 
-// Triangular factors of one level as a sequence of "chunks" per block: the L
-// chunks of a block in wavefront (level-set) order, then its U chunks.  A
-// chunk holds <= kChunkRows independent rows of one wavefront and is one
-// contiguous, 16-byte aligned byte range of <= StageBytesOf<VT> bytes:
-//   int32 {nrows, S, upper, more}     S = entry slots per row; more = 1 when
-//                                     another slice of the same layout follows
-//                                     in the same chunk (FP32: up to kMaxSlices
-//                                     consecutive wavefront slices per chunk
-//                                     when they fit)
+// ---- factor stream of the single-system substitutions ------------------------------
+// Every block's factors as a sequence of slices in wavefront (level-set) order,
+// those of L before those of U; a slice holds independent rows of one wavefront,
+// longest first.  Slices are packed into items; item g of a block is one bulk
+// copy into ring slot g % slots, and is read by consumer g % consumers (slots is a
+// multiple of consumers, so that a slot has one reader).
+// Values are -t_ij (L) and -u_ij/u_ii (U), formed in FP64 and rounded once, so
+// that a row is x_i = x_i d_i + sum_j v_ij x_j with d_i = 1 (L) or 1/u_ii (U);
+// rows and columns are byte offsets into the block's vector.
+//
+// FP32: x_i = fma(x_i, d_i, a0 + a1), a0 the sum of the even entries and of
+// those from 16 on, a1 that of the odd ones below 16, in order; one lane per row,
+// slices of at most 32 rows.  {row, d}[rows], padded to 16 bytes, then
+// row_bytes(np) per row: np pairs of entries (column, value), absent ones (0, 0).
+// Levels whose rows have at most 16 entries: an item is a group of four slices of
+// one factor, four int32 {rows - 1, offset in the high half}, then the slices; four
+// consumer warps.  L's records end with the row's last pair; U's hold the pairs in
+// reverse.  So the entries of the slice just before, the nearest columns, sit in
+// the last kLatePairs pairs: a slice of one row at kNoRow separates slices that
+// need more, and L from U, and fills a factor's last group.
+// Levels with longer rows (np = kLongRows): one slice per item, one consumer
+// warp; header int32 {rows - 1, 0, z, 0}, the slice with np = 8, and {column,
+// value}[z][rows] for the entries from 16 on (absent: column -1).
+//
+// FP64 and complex: four lanes per row, a row's entry e in lane e % 4; lane
+// sums start from x_i in lane 0 and use two chains (entries 0, 2, 4, ... and 1,
+// 3 of the lane); the row is (s0 + s1) + (s2 + s3).  A consumer is a set of four
+// warps, a slice at most 32 rows; slice k of the block belongs to consumer k %
+// consumers, an item holds several slices of one consumer.  Slice header int32
+// {rows - 1, distance to the next slice of the item (0: none), z, flags}; z =
+// entries of the longest row.  Per lane (lane_bytes): VT v[np], int32 c[np], int32
+// row (absent: 0, 0); then {VT v, int32 c, pad}[.][4 rows] for the lanes' entries
+// from 4 on.  The products x_i / u_ii are formed for the whole block between L
+// and U by kLaneScale slices (VT d[rows], z: first row; an item of its own).  The
+// slices of an item have the same class.  kSync: the slice ends its wavefront;
+// bits 24 and up: number of wavefronts that end in the other consumers' slices
+// since this consumer's last one.
+// Records are an odd number of 16-byte words, so that 16-byte shared loads of
+// consecutive records touch every bank once.
+constexpr int kStageBytes = 4096;               // batched substitutions: largest chunk
+constexpr int kRingData = 64 * 1024;
+constexpr int kMaxSlots = kRingData / kStageBytes;
+constexpr int kRingBytes = kRingData + 2 * kMaxSlots * 8 + 64;   // ring + mbarriers + flags
+constexpr int kItemHeader = 16;
+constexpr int kMaxItemBytes = 16192;            // head and a slot for each of four consumers within kRingBytes
+constexpr int kItemDepth = 16;                  // most slots per consumer
+constexpr int kLatePairs = 3;
+constexpr int kNoRow = -4;
+constexpr int kLaneItemBytes = 8192;            // FP64: slices of a consumer are joined into items of about this size
+constexpr int kLongRows = 16;
+enum { kSync = 1 };
+// class of a slice (flags >> kLaneShift & 7): longest row 1, 2, up to 4 entries, more, more than 16; scaling
+enum { kLaneShift = 4, kLane1 = 0, kLane2, kLane4, kLaneFull, kLaneLong, kLaneScale };
+template <typename VT> struct OneLaneRows { static constexpr bool value = false; };
+template <> struct OneLaneRows<float> { static constexpr bool value = true; };
+__host__ __device__ constexpr int odd16(int bytes) { return (((bytes + 15) / 16) | 1) * 16; }
+__host__ __device__ constexpr int row_bytes(int np) { return odd16(16 * np); }
+template <typename VT>
+__host__ __device__ constexpr int lane_bytes(int kq) { return odd16(kq * ((int)sizeof(VT) + 4) + 4); }
+
+// Start of a substitution CTA's shared memory: the ring's barriers and the flag
+// that ends every wait of the CTA; the block's vector and the ring follow.
+struct StreamHead {
+    uint64_t full[4 * kItemDepth], empty[4 * kItemDepth];
+    int abort_flag, pad[3];
+};
+static_assert(sizeof(StreamHead) % 16 == 0 && (int)sizeof(StreamHead) + 4 * kMaxItemBytes <= kRingBytes, "smallest ring");
+
+struct StreamView {
+    const unsigned char *data;
+    const int64_t *off;        // items + 1 byte offsets into data
+    const int32_t *blk_item;   // nblk + 1 item range of every block
+    const int32_t *split;      // nblk: items of L (FP32), slices with kSync (FP64)
+    int32_t np;                // pairs per row record (FP32), entries per lane record (FP64)
+    int32_t consumers;         // FP32: 4, 1 for long rows; FP64: 2 or 4
+    int32_t slots, slot_bytes; // the ring
+};
+
+// ---- chunks of the batched substitutions --------------------------------------------
+// Per block the L chunks in wavefront order, then the U chunks.  A chunk holds
+// independent rows of one wavefront and is one contiguous, 16-byte aligned byte
+// range of at most kStageBytes bytes:
+//   int32 {nrows, S, upper, 0}        S = entry slots per row
 //   int32 rows[pad4(nrows)]           block-local row of every slot
 //   int32 lens[pad4(nrows)]           entries of every slot
-//   int32 cols[pad4(S*nrows)]         block-local columns
-//   VT    vals[S*nrows] padded to 16 bytes: -t_ij in L chunks, -u_ij/u_ii in
-//         U chunks (formed in FP64, rounded once), so that a row is
-//         x_i = x_i * d_i + sum_j vals_ij x_j with d_i = 1 (L) or 1/u_ii (U)
-//   VT    dinv[nrows]  padded to 16 bytes (U chunks: 1/u_ii)
-// Entry q of row slot t sits at
-//   FP32 (one lane per row, S = maxlen):          q*nrows + t
-//   FP64 (four lanes per row, S = 4*ceil(maxlen/4)): ((q/4)*nrows + t)*4 + q%4
-// so a warp always reads consecutive addresses.  The chunks of a block move
-// into a shared-memory ring of kRingData bytes CPG at a time: group g (chunks
-// CPG*g onwards, contiguous in global memory) is one bulk copy into ring slot
-// g % (kRingData / (CPG*StageBytesOf<VT>)), and a chunk is found in its slot by
-// skipping the chunks before it (their sizes follow from their headers).
-// The FP32 substitutions move kGroupChunks chunks per copy (one per consumer
-// warp); the FP64 and batched ones, whose warps share every chunk, move one.
-constexpr int kStageBytes = 4096;
-constexpr int kGroupChunks = 4;
-constexpr int kRingData = 16 * kStageBytes;
-constexpr int kMaxSlots = kRingData / kStageBytes;
-constexpr int kConsumerWarps = 4;
-constexpr int kChunkRows = 32;
-constexpr int kTrsvThreads2 = 32 * (kConsumerWarps + 1);
-constexpr int kRingBytes = kRingData + 2 * kMaxSlots * 8 + 64;   // ring + mbarriers + flags
-template <typename VT> struct LanesPerRow { static constexpr int value = 4; };
-template <> struct LanesPerRow<float> { static constexpr int value = 1; };
-// Largest chunk of a value type: complex chunks (16-byte values) are twice as
-// large, so that a typical wavefront still fits in one chunk (one hand-off).
-template <typename VT> struct StageBytesOf { static constexpr int value = kStageBytes; };
-template <> struct StageBytesOf<zc> { static constexpr int value = 2 * kStageBytes; };
-// FP32 chunks (single system) hold up to kMaxSlices consecutive wavefront
-// slices in 8 KB, so that a consumer warp hands the sweep on once per four
-// wavefronts (a hand-off costs more than a slice solved by the same warp).
-template <> struct StageBytesOf<float> { static constexpr int value = 2 * kStageBytes; };
-constexpr int kMaxSlices = 4;
-
+//   int32 cols[pad4(S*nrows)]         block-local columns, entry q of slot t at q*nrows + t
+//   float vals[pad4(S*nrows)]         as in the stream above
+//   float dinv[pad4(nrows)]           U chunks: 1/u_ii
+// Chunk k of a block is one bulk copy into ring slot k % kMaxSlots.
 struct ChunkView {
     const unsigned char *data;
     const int64_t *off;        // nchunk + 1 byte offsets into data
@@ -73,9 +115,8 @@ struct LevelView {
     int64_t s, e;              // rows [s, e) of the multilevel order
     int64_t stail;             // n - e
     int32_t nblk;
-    int32_t max_slots;         // longest chunk row (entry slots) of the level's factors
     const int64_t *blk_row;    // nblk + 1, level-local
-    ChunkView C;               // L and U of every block (see above)
+    StreamView S;              // L and U of every block (see above)
     int32_t *err;              // device error word (1: a bounded wait expired)
     const int64_t *F_rp;       // d rows
     const int32_t *F_ci;       // global column (>= e)

@@ -1,0 +1,98 @@
+"""Block substitutions at the edges of their variants: record sizes, slices and
+groups that are full, partial or empty, rows longer than the records, wide and
+one-row wavefronts, vectors in shared and in global memory.
+
+The handle is built from random triangular factors (no coupling, no
+correction), so one application is U^-1 L^-1 r per block, compared with plain
+FP64 substitutions.  The off-diagonal row sums are at most 1/2 and the
+diagonals in [1, 2]: each triangular inverse has infinity norm at most 2, a row of
+m entries is summed with a relative error of at most (m + 3) eps, and so two
+solves stay within 8 (m + 3) eps of the largest component; with m <= 40 that
+is 4e-14 in FP64 and 2.1e-5 in FP32 (FP32 factors and right-hand side: 4 eps
+more).
+"""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+import gemslr_inputs as gi
+from oracle.ilu import lu_solve
+
+pytestmark = pytest.mark.gpu
+
+# name: (rows of every block, most entries per row, band, chain: every row needs the one before)
+CASES = {
+    "one_row": ([1, 2, 3], 2, 4, False),
+    "two_entries": ([33, 257, 130], 2, 60, False),
+    "six_entries": ([31, 200, 700], 6, 90, False),
+    "ten_entries": ([64, 1000, 5000], 10, 300, False),
+    "near_ten": ([97, 600], 10, 12, True),            # many entries from the slice just before
+    "sixteen_entries": ([500, 129], 16, 400, False),
+    "seventeen_entries": ([500, 40], 17, 100, False),
+    "forty_entries": ([400, 350], 40, 200, False),
+    "chain": ([300, 45], 3, 5, True),                 # one row per wavefront
+    "no_lower": ([200, 70], 0, 50, False),
+    "wide": ([6000, 5000], 3, 6000, False),           # wavefronts of hundreds of rows
+    "global_vector": ([46000, 300], 2, 9000, False),  # beyond shared memory in every precision
+}
+
+
+def _triangles(rng, n, most, band, chain, cplx):
+    """Strictly lower L and upper U (diagonal included) with the stated patterns."""
+    val = (lambda k: rng.uniform(-1, 1, k) + 1j * rng.uniform(-1, 1, k)) if cplx else (lambda k: rng.uniform(-1, 1, k))
+    out = []
+    for up in (False, True):
+        ptr, ind, dat = [0], [], []
+        for i in range(n):
+            room = min(band, n - 1 - i if up else i)
+            k = min(int(rng.integers(0, most + 1)), room)
+            off = set(rng.choice(room, size=k, replace=False) + 1) if k else set()
+            if chain and room and most:
+                off = set(list(off)[: most - 1]) | {1}
+            cols = sorted(i + o if up else i - o for o in off)
+            v = val(len(cols))
+            v = v * (0.5 / max(np.abs(v).sum(), 0.5)) if len(cols) else v
+            if up:
+                d = rng.uniform(1, 2)
+                cols, v = [i] + cols, np.concatenate([[d], v * d])
+            ind += cols
+            dat.append(v)
+            ptr.append(len(ind))
+        dat = np.concatenate(dat) if ind else np.zeros(0)
+        out.append(sp.csr_matrix((dat, np.array(ind, dtype=np.int32), ptr), shape=(n, n)))
+    return out
+
+
+@pytest.mark.parametrize("kind", ["fp64", "mixed", "complex"])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_substitutions_against_plain_solves(name, kind):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_03224_gb300 import Gemslr
+    sizes, most, band, chain = CASES[name]
+    cplx = kind == "complex"
+    rng = np.random.default_rng(len(name) + most)
+    blocks = [_triangles(rng, n, most, band, chain, cplx) for n in sizes]
+    d, tail = sum(sizes), 5
+    n = d + tail
+    eye = sp.identity(tail, format="csr", dtype=complex if cplx else float)
+    zero = sp.csr_matrix((tail, tail), dtype=complex if cplx else float)
+    fac = dict(levels=[dict(s=0, e=d, L=sp.block_diag([b[0] for b in blocks], format="csr"),
+                            U=sp.block_diag([b[1] for b in blocks], format="csr"),
+                            E=sp.csr_matrix((tail, d)), F=sp.csr_matrix((d, tail)),
+                            W=np.zeros((tail, 0)), H=np.zeros((0, 0)))], last=dict(L=zero, U=eye))
+    A = gi.CSR(n, np.arange(n + 1), np.arange(n), np.ones(n))
+    part = dict(perm=np.arange(n, dtype=np.int32), level_ptr=np.array([0, d, n], dtype=np.int64),
+                nblk=np.array([len(sizes), 1], dtype=np.int32),
+                block_ptr=np.concatenate([np.cumsum([0] + sizes), [0, tail]]).astype(np.int64))
+    G = Gemslr.from_factors(A, part, fac, precision="mixed" if kind == "mixed" else "fp64")
+    r = rng.uniform(-1, 1, n) + (1j * rng.uniform(-1, 1, n) if cplx else 0)
+    z = G.apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    ref = r.copy()
+    o = 0
+    for (L, U), m in zip(blocks, sizes):
+        ref[o:o + m] = lu_solve(L, U, r[o:o + m])
+        o += m
+    tol = 3e-5 if kind == "mixed" else 1e-13
+    assert np.max(np.abs(z - ref)) <= tol * np.max(np.abs(ref)), np.max(np.abs(z - ref))
