@@ -433,7 +433,7 @@ void append_lanes(const Csr &T, int64_t r0, const Waves &W, bool upper, int np, 
     auto bytes = [&](int64_t n, int64_t m) {
         return kItemHeader + (size_t)(4 * n) * (lb + (size_t)std::max<int64_t>(0, (m + 3) / 4 - 4) * tb);
     };
-    for (const SliceRows &s : cut_slices<VT>(W, r0, upper, 32)) {
+    for (const SliceRows &s : cut_slices<VT>(W, r0, upper, kLaneRows<VT>)) {
         for (int64_t at = 0; at < s.n;) {
             int64_t n = 1;
             while (at + n < s.n && bytes(n + 1, s.longest) <= (size_t)kMaxItemBytes) ++n;
@@ -548,7 +548,7 @@ void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, St
     out.np = trsv_record(one, longest);
     int64_t nwave = 1;
     for (size_t b = 0; b < nb; ++b) nwave += (int64_t)(wl[b].ptr.size() + wu[b].ptr.size());
-    out.consumers = !one ? trsv_sets((double)(2 * bp.back()) / (double)nwave) : out.np == kLongRows ? 1 : 4;
+    out.consumers = !one ? trsv_sets((double)(2 * bp.back()) / (double)(nwave * kLaneRows<VT>)) : out.np == kLongRows ? 1 : 4;
     for (size_t b = 0; b < nb; ++b) {
         const int64_t r0 = bp[b];
         if constexpr (one) {

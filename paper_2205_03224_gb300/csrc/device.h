@@ -40,9 +40,9 @@ void launch_trsv(const LevelView<VT, WT> &lv, int mode, int smem_rows, const IoT
                  const PendingLowRank<VT, WT> &pl = PendingLowRank<VT, WT>());
 template <typename VT, typename WT> void set_trsv_smem_limit(int bytes);
 // the kernel variant of a level: StreamView::np for its longest row; sets of
-// warps (FP64) for its mean rows per wavefront
+// warps (FP64) for its mean slices per wavefront
 int trsv_record(bool one_lane, int longest);
-int trsv_sets(double width);
+int trsv_sets(double slices);
 template <typename VT, typename WT>
 void launch_couple(const LevelView<VT, WT> &lv, const IoT<VT> *in, VT *work, VT *partial, unsigned *counter,
                    VT *u, cudaStream_t st, const PendingLowRank<VT, WT> &pl = PendingLowRank<VT, WT>());

@@ -38,10 +38,11 @@ constexpr int kMaxCols = 160;     // Krylov columns per Gram-Schmidt pass (m + 1
 // warp; header int32 {rows - 1, 0, z, 0}, the slice with np = 8, and {column,
 // value}[z][rows] for the entries from 16 on (absent: column -1).
 //
-// FP64 and complex: four lanes per row, a row's entry e in lane e % 4; lane
+// FP64 and complex: four chains per row, a row's entry e in chain e % 4 (a lane;
+// two in complex arithmetic); chain
 // sums start from x_i in lane 0 and use two chains (entries 0, 2, 4, ... and 1,
 // 3 of the lane); the row is (s0 + s1) + (s2 + s3).  A consumer is a set of four
-// warps, a slice at most 32 rows; slice k of the block belongs to consumer k %
+// warps, a slice at most kLaneRows rows; slice k of the block belongs to consumer k %
 // consumers, an item holds several slices of one consumer.  Slice header int32
 // {rows - 1, distance to the next slice of the item (0: none), z, flags}; z =
 // entries of the longest row.  Per lane (lane_bytes): VT v[np], int32 c[np], int32
@@ -58,6 +59,7 @@ constexpr int kRingData = 64 * 1024;
 constexpr int kMaxSlots = kRingData / kStageBytes;
 constexpr int kRingBytes = kRingData + 2 * kMaxSlots * 8 + 64;   // ring + mbarriers + flags
 constexpr int kItemHeader = 16;
+template <typename VT> constexpr int kLaneRows = sizeof(VT) == 8 ? 32 : 16;   // rows per slice, FP64 and complex
 constexpr int kMaxItemBytes = 16192;            // head and a slot for each of four consumers within kRingBytes
 constexpr int kItemDepth = 16;                  // most slots per consumer
 constexpr int kLatePairs = 3;

@@ -114,6 +114,13 @@ struct BlockVec<VT, true> {
     __device__ __forceinline__ void store(int off, VT v) const {
         *reinterpret_cast<VT *>(reinterpret_cast<unsigned char *>(vec()) + off) = v;
     }
+    // component `part` of an FP64 or complex entry
+    __device__ __forceinline__ double part(int off, int part) const {
+        return *reinterpret_cast<const double *>(reinterpret_cast<const unsigned char *>(vec()) + off + 8 * part);
+    }
+    __device__ __forceinline__ void store_part(int off, int part, double v) const {
+        *reinterpret_cast<double *>(reinterpret_cast<unsigned char *>(vec()) + off + 8 * part) = v;
+    }
 };
 template <typename VT>
 struct BlockVec<VT, false> {
@@ -122,6 +129,12 @@ struct BlockVec<VT, false> {
     __device__ __forceinline__ VT load(int off) const { return *reinterpret_cast<const VT *>(base + max(off, 0)); }
     __device__ __forceinline__ void store(int off, VT v) const {
         if (off >= 0) *reinterpret_cast<VT *>(base + off) = v;
+    }
+    __device__ __forceinline__ double part(int off, int part) const {
+        return *reinterpret_cast<const double *>(base + off + 8 * part);
+    }
+    __device__ __forceinline__ void store_part(int off, int part, double v) const {
+        *reinterpret_cast<double *>(base + off + 8 * part) = v;
     }
 };
 

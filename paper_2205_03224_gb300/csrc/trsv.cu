@@ -26,7 +26,12 @@ namespace {
 // with few entries a compiler would, and the result would depend on the variant.
 __device__ __forceinline__ float sum_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double sum_rn(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ zc sum_rn(zc a, zc b) { return zc(__dadd_rn(a.re, b.re), __dadd_rn(a.im, b.im)); }
+
+// A product in the rounding of LaneMath.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ zc mul_rn(zc a, zc b) {
+    return zc(__fma_rn(a.re, b.re, -__dmul_rn(a.im, b.im)), __fma_rn(a.im, b.re, __dmul_rn(a.re, b.im)));
+}
 
 // ---- FP32 rows -----------------------------------------------------------------------
 // A row in registers: byte offset of x_i, d_i, and NP pairs of entries (byte
@@ -169,11 +174,8 @@ struct RowF64 {
     int w[4 * kUsed];
     __device__ __forceinline__ int col(int k) const { return w[kV * KQ + k]; }
     __device__ __forceinline__ int row() const { return w[(kV + 1) * KQ]; }
-    __device__ __forceinline__ VT val(int k) const {
-        const double a = __hiloint2double(w[kV * k + 1], w[kV * k]);
-        if constexpr (IsComplex<VT>::value) return zc(a, __hiloint2double(w[kV * k + 3], w[kV * k + 2]));
-        else return a;
-    }
+    __device__ __forceinline__ double val(int k) const { return __hiloint2double(w[kV * k + 1], w[kV * k]); }
+    __device__ __forceinline__ double imag(int k) const { return __hiloint2double(w[kV * k + 3], w[kV * k + 2]); }
 };
 
 template <typename VT, int KQ>
@@ -196,18 +198,43 @@ __device__ __forceinline__ void wavefront_end(int on) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %0, 0;\n\t@p bar.sync 2, %1;\n\t}" ::"r"(on), "n"(NT) : "memory");
 }
 
+// One lane's arithmetic.  FP64: v x by one FMA into the sum.  Complex: a lane
+// holds one component (im: the imaginary one) of its chain, v x rounded as
+// fma(v_re, x_re, -(v_im x_im)) and fma(v_im, x_re, v_re x_im), then added, so
+// that an entry costs a lane three FP64 instructions instead of six.
+template <typename VT, int KQ>
+struct LaneMath {
+    const RowF64<VT, KQ> &R;
+    bool im;
+    __device__ __forceinline__ double product(double re, double imag, VT x) const {
+        if constexpr (IsComplex<VT>::value) {
+            const double m = __dmul_rn(im ? re : imag, x.im);
+            return __fma_rn(im ? imag : re, x.re, im ? m : -m);
+        } else {
+            return __dmul_rn(re, x);
+        }
+    }
+    __device__ __forceinline__ double mul(int k, VT x) const { return product(R.val(k), R.imag(k), x); }
+    __device__ __forceinline__ double add(double a, double re, double imag, VT x) const {
+        if constexpr (IsComplex<VT>::value) return __dadd_rn(a, product(re, imag, x));
+        else return __fma_rn(re, x, a);
+    }
+    __device__ __forceinline__ double add(double a, int k, VT x) const { return add(a, R.val(k), R.imag(k), x); }
+};
+
 // The slices of one item, all of class C (see kernels.cuh), by the four warps of
-// a set.  Nothing but the loop itself is conditional: row slots past the last
-// repeat it without storing.
+// a set: four lanes per row, eight in complex arithmetic (two per chain lane).
+// Nothing but the loop itself is conditional: row slots past the last repeat it
+// without storing.
 template <int C, int KQ, int NS, typename VT, typename X>
 __device__ __forceinline__ void lane_slices(uint32_t p, const X &x, int warp, int lane, int &nsync) {
-    constexpr int NT = 128 * NS;
-    const int r4 = 8 * (warp % 4) + (lane >> 2), sub = lane & 3;
+    constexpr int NT = 128 * NS, kParts = IsComplex<VT>::value ? 2 : 1;      // lanes per chain lane
+    const int slot = (8 * (warp % 4) + (lane >> 2)) / kParts, sub = (lane / kParts) & 3, part = lane & (kParts - 1);
     RowF64<VT, KQ> A, B;
     int4 h = lds<int4>(p);
-    fetch_f64(p, min(r4, h.x), sub, A);
+    fetch_f64(p, min(slot, h.x), sub, A);
     auto step = [&](const RowF64<VT, KQ> &R, RowF64<VT, KQ> &next) {
-        const int t = min(r4, h.x), before = h.w >> 24, after = h.w & kSync;
+        const int t = min(slot, h.x), before = h.w >> 24, after = h.w & kSync;
         const uint32_t pn = p + h.y;
         const int4 hn = lds<int4>(pn);
 #pragma unroll
@@ -217,33 +244,32 @@ __device__ __forceinline__ void lane_slices(uint32_t p, const X &x, int warp, in
         VT xq[kUse];
 #pragma unroll
         for (int k = 0; k < kUse; ++k) xq[k] = x.load(R.col(k));
-        const VT self = x.load(R.row());
-        VT a0 = sub == 0 ? self : (VT)0;
+        const double self = x.part(R.row(), part);
+        const LaneMath<VT, KQ> M{R, part != 0};
+        double a0 = M.add(sub == 0 ? self : 0.0, 0, xq[0]);
         if constexpr (C < kLaneFull) {
-            a0 += R.val(0) * xq[0];
-            if constexpr (C >= kLane2) a0 += shfl_xor(a0, 1);
-            if constexpr (C >= kLane4) a0 += shfl_xor(a0, 2);
+            if constexpr (C >= kLane2) a0 += shfl_xor(a0, kParts);
+            if constexpr (C >= kLane4) a0 += shfl_xor(a0, 2 * kParts);
         } else {
-            VT a1 = R.val(1) * xq[1];
-            a0 += R.val(0) * xq[0];
-            if constexpr (KQ > 3) a1 += R.val(3) * xq[3];
-            if constexpr (KQ > 2) a0 += R.val(2) * xq[2];
+            double a1 = M.mul(1, xq[1]);
+            if constexpr (KQ > 3) a1 = M.add(a1, 3, xq[3]);
+            if constexpr (KQ > 2) a0 = M.add(a0, 2, xq[2]);
             if constexpr (C == kLaneLong) {     // the rest of long rows, from the staged slice
                 constexpr int kRest = ((int)sizeof(VT) + 4 + 15) / 16 * 16;
                 const int n4 = 4 * (h.x + 1);
                 uint32_t r = p + kItemHeader + lane_bytes<VT>(KQ) * n4 + kRest * (4 * t + sub);
                 for (int k = 4; k < (h.z + 3) >> 2; ++k, r += kRest * n4)
-                    a0 += lds<VT>(r) * x.load(lds<int>(r + (uint32_t)sizeof(VT)));
+                    a0 = M.add(a0, lds<double>(r), kParts > 1 ? lds<double>(r + 8) : 0.0, x.load(lds<int>(r + (uint32_t)sizeof(VT))));
             }
             a0 = sum_rn(a0, a1);
-            a0 += shfl_xor(a0, 1);
-            a0 += shfl_xor(a0, 2);
+            a0 += shfl_xor(a0, kParts);
+            a0 += shfl_xor(a0, 2 * kParts);
         }
-        if (sub == 0 && r4 == t) x.store(R.row(), a0);
+        if (sub == 0 && slot == t) x.store_part(R.row(), part, a0);
         const bool more = h.y != 0;
         p = pn;
         h = hn;
-        fetch_f64(p, min(r4, h.x), sub, next);  // before the barrier: in flight while the others come to it
+        fetch_f64(p, min(slot, h.x), sub, next);    // before the barrier: in flight while the others come to it
         wavefront_end<NT>(after);
         return more;
     };
@@ -276,7 +302,7 @@ __device__ __forceinline__ void consume_lanes(ItemWalk &W, const X &x, int warp,
                 for (int k = h.w >> 24; k > 0; --k, --nsync) wavefront_end<NT>(1);
                 for (int i = 32 * (warp % 4) + lane; i <= h.x; i += 128) {
                     const int a = (h.z + i) * (int)sizeof(VT);
-                    x.store(a, x.load(a) * lds<VT>(p + kItemHeader + i * (int)sizeof(VT)));
+                    x.store(a, mul_rn(x.load(a), lds<VT>(p + kItemHeader + i * (int)sizeof(VT))));
                 }
                 wavefront_end<NT>(h.w & kSync);
                 nsync -= h.w & kSync;
@@ -468,7 +494,7 @@ int trsv_record(bool one_lane, int longest) {
     if (one_lane) return longest <= 2 ? 1 : longest <= 6 ? 3 : longest <= 10 ? 5 : longest <= 16 ? 8 : kLongRows;
     return longest <= 4 ? 1 : longest <= 8 ? 2 : longest <= 12 ? 3 : 4;
 }
-int trsv_sets(double width) { return width > 48.0 ? 4 : 2; }
+int trsv_sets(double slices) { return slices > 1.5 ? 4 : 2; }
 
 template <typename VT, typename WT>
 void launch_trsv(const LevelView<VT, WT> &lv, int mode, int smem_rows, const IoT<VT> *in, VT *work,
