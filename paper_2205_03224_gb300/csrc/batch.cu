@@ -23,6 +23,9 @@ namespace gemslr {
 void launch_btrsv(const BatchLevel &lv, int mode, int rpc, size_t smem_bytes, const double *in, float *work,
                   double *out_final, float *scratch, cudaStream_t st);
 void set_btrsv_smem_limit(int bytes);
+void launch_bstream(const BatchLevel &lv, const BatchUnits &u, int mode, const double *in, float *work, double *out_final,
+                    cudaStream_t st);
+size_t bstream_smem(int64_t rows, int rpc, const StreamView &S);
 void launch_bcouple(const BatchLevel &lv, const double *in, float *work, cudaStream_t st);
 void launch_blowrank(const BatchLevel &lv, float *work, cudaStream_t st);
 void launch_bspmv(int64_t nrows, const int64_t *rp, const int32_t *ci, const double *v, const double *x,
@@ -57,7 +60,9 @@ struct BLevelHost {          // device level plus what the launcher needs
     int rpc = 0;              // right-hand sides per substitution CTA (0: vector in global memory)
     size_t smem_bytes = 0;
     int64_t rows = 0;         // rows of the level's blocks, all systems
-    int64_t l_bytes = 0, u_bytes = 0;   // stored L and U chunks
+    int64_t l_bytes = 0, u_bytes = 0;   // stored L and U
+    bool streamed = false;
+    std::vector<BatchUnits> units;      // streamed level: its launches
     int64_t f_nnz = 0;        // nonzeros of F
 };
 
@@ -82,6 +87,10 @@ struct gemslr_batch_ctx {
     int m_alloc = 0;
     double *V = nullptr, *Z = nullptr, *w = nullptr, *x = nullptr, *b = nullptr, *r = nullptr, *vin = nullptr,
            *zout = nullptr;
+    // a level's groups of units run side by side: side streams forked from and
+    // joined back into the caller's stream within every sweep
+    cudaStream_t side[kBatchStreams - 1] = {};
+    cudaEvent_t ev_fork = nullptr, ev_join[kBatchStreams - 1] = {};
     // graphs
     cudaStream_t cap = nullptr;
     cudaGraphExec_t apply_exec = nullptr, solve_exec = nullptr;
@@ -98,6 +107,11 @@ struct gemslr_batch_ctx {
         if (solve_exec) cudaGraphExecDestroy(solve_exec);
         if (solve_graph) cudaGraphDestroy(solve_graph);
         if (cap) cudaStreamDestroy(cap);
+        for (cudaStream_t t : side)
+            if (t) cudaStreamDestroy(t);
+        if (ev_fork) cudaEventDestroy(ev_fork);
+        for (cudaEvent_t e : ev_join)
+            if (e) cudaEventDestroy(e);
     }
 };
 
@@ -128,12 +142,103 @@ int dev_smem_optin() {
     return b;
 }
 
-// Start row of level l of system s inside the batch, its blocks, E/F/W.
-void build_batch_level(gemslr_batch_ctx *B, int l, bool last, int rows_cta, BLevelHost &out) {
+// The substitutions of one level as streams, if every block's vector fits in
+// shared memory (for all right-hand sides, or for half of them) and no row has
+// more than 16 entries.  A unit's CTA holds its vector, so units are launched in
+// groups by the number of them that fit on an SM, the largest first, and within a
+// group the blocks with the most items first (no long block in the last wave).
+bool build_streams(gemslr_batch_ctx *B, int l, bool last, const std::vector<int32_t> &blk_nr, BLevelHost &out) {
+    StreamHost sh;
+    int64_t longest = 0;
+    auto level = [&](int s) -> const HostLevel & { return last ? B->sys[s].last : B->sys[s].lev[l]; };
+    for (int s = 0; s < B->nsys; ++s)
+        for (const Csr *T : {&level(s).L, &level(s).U})
+            for (int64_t i = 0; i < T->nrows; ++i)
+                longest = std::max(longest, T->rp[i + 1] - T->rp[i] - (T == &level(s).U ? 1 : 0));
+    sh.np = trsv_record(true, (int)longest);
+    sh.consumers = kBatchSets;
+    if (sh.np == kLongRows) return false;
+    int64_t lb = 0, ub = 0;
+    for (int s = 0; s < B->nsys; ++s)
+        append_batch_stream(level(s).L, level(s).U, level(s).bp, kBatchSliceRows, kBatchItemBytes, sh, lb, ub);
+    StreamView &S = out.v.S;
+    S.np = sh.np;
+    S.consumers = sh.consumers;
+    S.slot_bytes = std::max(sh.slot_bytes, 128);
+    S.slots = kBatchSets * kBatchDepth;
+    int dev = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    const size_t optin = (size_t)dev_smem_optin();
+    struct Unit { int32_t blk, rhs0, rpc, fit, items; };
+    std::vector<Unit> all;
+    for (size_t b = 0; b < blk_nr.size(); ++b) {
+        if (blk_nr[b] == 0) continue;
+        int rpc = kBatchRhs;
+        if (bstream_smem(blk_nr[b], rpc, S) > optin) rpc /= 2;
+        const size_t bytes = bstream_smem(blk_nr[b], rpc, S);
+        if (bytes > optin) return false;
+        const int fit = (int)std::min<size_t>(4, per_sm / (bytes + 1024));
+        for (int r = 0; r < kBatchRhs; r += rpc) all.push_back({(int32_t)b, r, rpc, fit, sh.blk_item[b + 1] - sh.blk_item[b]});
+    }
+    std::stable_sort(all.begin(), all.end(), [](const Unit &x, const Unit &y) {
+        return x.fit != y.fit ? x.fit < y.fit : x.rpc != y.rpc ? x.rpc < y.rpc : x.items > y.items;
+    });
+    Arena &a = B->arena;
+    S.data = a.upload(sh.data);
+    S.off = a.upload(sh.off);
+    S.blk_item = a.upload(sh.blk_item);
+    S.split = a.upload(sh.split);
+    out.units.clear();
+    for (size_t i = 0; i < all.size();) {
+        BatchUnits u;
+        u.rpc = all[i].rpc;
+        std::vector<int32_t> blk, rhs0;
+        for (const int fit = all[i].fit; i < all.size() && all[i].fit == fit && all[i].rpc == u.rpc; ++i) {
+            blk.push_back(all[i].blk);
+            rhs0.push_back(all[i].rhs0);
+            u.smem = std::max(u.smem, bstream_smem(blk_nr[all[i].blk], u.rpc, S));
+        }
+        u.n = (int32_t)blk.size();
+        u.blk = a.upload(blk);
+        u.rhs0 = a.upload(rhs0);
+        out.units.push_back(u);
+    }
+    out.rpc = kBatchRhs;
+    for (const Unit &u : all) out.rpc = std::min(out.rpc, (int)u.rpc);
+    out.l_bytes = lb;
+    out.u_bytes = ub;
+    out.streamed = true;
+    return true;
+}
+
+// Level l of every system: blocks, substitution data, E/F/W.  With lists_only the
+// level exists already and only the coupling kernels' work list changes.
+void build_batch_level(gemslr_batch_ctx *B, int l, bool last, int rows_cta, BLevelHost &out, bool lists_only = false) {
+    if (lists_only) {
+        std::vector<int32_t> cta_seg, seg_cta0{0};
+        std::vector<int64_t> cta_i0;
+        for (int s = 0; s < B->nsys; ++s) {
+            const int64_t len = B->sys[s].n - B->sys[s].lev[l].e;
+            for (int64_t i0 = 0; i0 < len; i0 += rows_cta) {
+                cta_seg.push_back(s);
+                cta_i0.push_back(i0);
+            }
+            seg_cta0.push_back((int32_t)cta_seg.size());
+        }
+        Arena &a = B->arena;
+        BatchLevel &v = out.v;
+        v.ncta = (int32_t)cta_seg.size();
+        v.rows_cta = rows_cta;
+        v.cta_seg = a.upload(cta_seg);
+        v.cta_i0 = a.upload(cta_i0);
+        v.seg_cta0 = a.upload(seg_cta0);
+        v.partial = (float *)a.alloc(sizeof(float) * std::max<int64_t>(1, v.ncta) * kBatchMaxRank * kBatchRhs);
+        return;
+    }
     ChunkHost ch;
     std::vector<int64_t> blk_r0, blk_f0, F_rp{0}, E_rp{0}, seg_r0, seg_len, seg_e0, seg_w0, seg_h0;
-    std::vector<int32_t> blk_nr, blk_sys, F_ci, E_ci, seg_k, cta_seg, seg_cta0{0};
-    std::vector<int64_t> cta_i0;
+    std::vector<int32_t> blk_nr, blk_sys, F_ci, E_ci, seg_k, F_rows, F_blk{0};
     std::vector<float> F_v, E_v, H;
     std::vector<__nv_bfloat16> W;
     int64_t frows = 0, maxrows = 0;
@@ -141,22 +246,16 @@ void build_batch_level(gemslr_batch_ctx *B, int l, bool last, int rows_cta, BLev
         const Hierarchy &h = B->sys[s];
         const HostLevel &hl = last ? h.last : h.lev[l];
         const int64_t bs = B->base[s];
-        ChunkHost cs;
-        build_chunks(hl.L, hl.U, hl.bp, cs, kBatchChunkRows);
-        // append chunk data with offsets shifted
-        const int64_t doff = (int64_t)ch.data.size();
-        const int64_t coff = (int64_t)ch.off.size() - 1;
-        ch.data.insert(ch.data.end(), cs.data.begin(), cs.data.end());
-        for (size_t q = 1; q < cs.off.size(); ++q) ch.off.push_back(cs.off[q] + doff);
-        // cs.data may carry a 16-byte filler when it has no chunks; keep offsets consistent
-        if (cs.off.size() == 1 && !cs.data.empty()) { /* filler bytes are never referenced */ }
         for (size_t j = 0; j + 1 < hl.bp.size(); ++j) {
             blk_r0.push_back(bs + hl.s + hl.bp[j]);
             blk_nr.push_back((int32_t)(hl.bp[j + 1] - hl.bp[j]));
             blk_sys.push_back(s);
             blk_f0.push_back(frows + hl.bp[j]);
             maxrows = std::max(maxrows, hl.bp[j + 1] - hl.bp[j]);
-            ch.blk_chunk.push_back((int32_t)(coff + cs.blk_chunk[j + 1]));
+            if (!last)
+                for (int64_t i = hl.bp[j]; i < hl.bp[j + 1]; ++i)
+                    if (hl.F.rp[i + 1] > hl.F.rp[i]) F_rows.push_back((int32_t)(i - hl.bp[j]));
+            F_blk.push_back((int32_t)F_rows.size());
         }
         if (!last) {
             for (int64_t i = 0; i < hl.F.nrows; ++i) {
@@ -183,69 +282,77 @@ void build_batch_level(gemslr_batch_ctx *B, int l, bool last, int rows_cta, BLev
             seg_h0.push_back((int64_t)H.size());
             for (double v : hl.W) W.push_back(__float2bfloat16_rn((float)v));
             for (double v : hl.H) H.push_back((float)v);
-            for (int64_t i0 = 0; i0 < len; i0 += rows_cta) {
-                cta_seg.push_back(s);
-                cta_i0.push_back(i0);
-            }
-            seg_cta0.push_back((int32_t)cta_seg.size());
         }
         frows += hl.e - hl.s;
     }
-    out.rows = out.l_bytes = out.u_bytes = 0;    // the level may be rebuilt (autotuning)
-    for (size_t c = 0; c + 1 < ch.off.size(); ++c) {
-        int32_t upper = 0;
-        std::memcpy(&upper, ch.data.data() + ch.off[c] + 8, 4);
-        (upper ? out.u_bytes : out.l_bytes) += ch.off[c + 1] - ch.off[c];
-    }
+    out.rows = out.l_bytes = out.u_bytes = 0;
     for (int32_t nr : blk_nr) out.rows += nr;
     out.f_nnz = (int64_t)F_ci.size();
-    if (ch.data.empty()) ch.data.resize(16, 0);
+    const bool streamed = build_streams(B, l, last, blk_nr, out);
+    if (!streamed) {
+        for (int s = 0; s < B->nsys; ++s) {
+            const HostLevel &hl = last ? B->sys[s].last : B->sys[s].lev[l];
+            build_chunks(hl.L, hl.U, hl.bp, ch, kBatchChunkRows);
+        }
+        for (size_t c = 0; c + 1 < ch.off.size(); ++c) {
+            int32_t upper = 0;
+            std::memcpy(&upper, ch.data.data() + ch.off[c] + 8, 4);
+            (upper ? out.u_bytes : out.l_bytes) += ch.off[c + 1] - ch.off[c];
+        }
+        if (ch.data.empty()) ch.data.resize(16, 0);
+    }
     Arena &a = B->arena;
     BatchLevel &v = out.v;
     v.nblk = (int32_t)blk_r0.size();
-    // CTAs are dispatched in index order and a block's time grows with its
-    // chunk count (one consumer barrier per chunk): the blocks with the most
-    // chunks go first, so that no long block starts in the last wave
-    std::vector<int32_t> order(v.nblk);
-    for (int32_t j = 0; j < v.nblk; ++j) order[j] = j;
-    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
-        return ch.blk_chunk[x + 1] - ch.blk_chunk[x] > ch.blk_chunk[y + 1] - ch.blk_chunk[y];
-    });
-    v.order = a.upload(order);
+    if (!streamed) {
+        // CTAs are dispatched in index order and a block's time grows with its
+        // chunk count (one consumer barrier per chunk): the blocks with the most
+        // chunks go first, so that no long block starts in the last wave
+        std::vector<int32_t> order(v.nblk);
+        for (int32_t j = 0; j < v.nblk; ++j) order[j] = j;
+        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+            return ch.blk_chunk[x + 1] - ch.blk_chunk[x] > ch.blk_chunk[y + 1] - ch.blk_chunk[y];
+        });
+        v.order = a.upload(order);
+    }
     v.blk_sys = a.upload(blk_sys);
     v.live = nullptr;
     v.final_up = (!last && l == 0) ? 1 : 0;
     v.blk_r0 = a.upload(blk_r0);
     v.blk_nr = a.upload(blk_nr);
     v.blk_f0 = a.upload(blk_f0);
-    v.C.data = a.upload(ch.data);
-    v.C.off = a.upload(ch.off);
-    v.C.blk_chunk = a.upload(ch.blk_chunk);
     v.err = B->err;
-    const int optin = dev_smem_optin();
-    // the most right-hand sides per CTA whose block vectors fit in shared
-    // memory; a split (fewer than kBatchRhs) multiplies the CTAs, and is taken
-    // only while they all fit on the GPU at once: otherwise the CTAs would run
-    // in many waves, slower than one wave with the vectors in global memory
-    out.rpc = 0;
-    out.smem_bytes = 0;
-    for (int rpc = kBatchRhs; rpc >= 1; rpc /= 2) {
-        const size_t bytes = (size_t)kRingBytes + (size_t)maxrows * rpc * sizeof(float);
-        if (bytes <= (size_t)optin) {
-            out.rpc = rpc;
-            out.smem_bytes = bytes;
-            break;
+    v.F_rows = a.upload(F_rows);
+    v.F_blk = a.upload(F_blk);
+    if (!streamed) {
+        v.C.data = a.upload(ch.data);
+        v.C.off = a.upload(ch.off);
+        v.C.blk_chunk = a.upload(ch.blk_chunk);
+        const int optin = dev_smem_optin();
+        // the most right-hand sides per CTA whose block vectors fit in shared
+        // memory; a split (fewer than kBatchRhs) multiplies the CTAs, and is taken
+        // only while they all fit on the GPU at once: otherwise the CTAs would run
+        // in many waves, slower than one wave with the vectors in global memory
+        out.rpc = 0;
+        out.smem_bytes = 0;
+        for (int rpc = kBatchRhs; rpc >= 1; rpc /= 2) {
+            const size_t bytes = (size_t)kRingBytes + (size_t)maxrows * rpc * sizeof(float);
+            if (bytes <= (size_t)optin) {
+                out.rpc = rpc;
+                out.smem_bytes = bytes;
+                break;
+            }
         }
-    }
-    if (out.rpc > 0 && out.rpc < kBatchRhs) {
-        int dev = 0, sms = 1, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        const int64_t resident = (int64_t)sms * std::max<int64_t>(1, per_sm / (int64_t)out.smem_bytes);
-        if ((int64_t)v.nblk * (kBatchRhs / out.rpc) > resident) {
-            out.rpc = 0;
-            out.smem_bytes = 0;
+        if (out.rpc > 0 && out.rpc < kBatchRhs) {
+            int dev = 0, sms = 1, per_sm = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+            const int64_t resident = (int64_t)sms * std::max<int64_t>(1, per_sm / (int64_t)out.smem_bytes);
+            if ((int64_t)v.nblk * (kBatchRhs / out.rpc) > resident) {
+                out.rpc = 0;
+                out.smem_bytes = 0;
+            }
         }
     }
     if (!last) {
@@ -264,15 +371,10 @@ void build_batch_level(gemslr_batch_ctx *B, int l, bool last, int rows_cta, BLev
         v.seg_h0 = a.upload(seg_h0);
         v.W = a.upload(W);
         v.H = a.upload(H);
-        v.ncta = (int32_t)cta_seg.size();
-        v.rows_cta = rows_cta;
-        v.cta_seg = a.upload(cta_seg);
-        v.cta_i0 = a.upload(cta_i0);
-        v.seg_cta0 = a.upload(seg_cta0);
         v.seg_counter = (unsigned *)a.alloc(sizeof(unsigned) * std::max(1, B->nsys));
         GEMSLR_CUDA(cudaMemset(v.seg_counter, 0, sizeof(unsigned) * std::max(1, B->nsys)));
-        v.partial = (float *)a.alloc(sizeof(float) * std::max<int64_t>(1, v.ncta) * kBatchMaxRank * kBatchRhs);
         v.u = (float *)a.alloc(sizeof(float) * std::max(1, B->nsys) * kBatchMaxRank * kBatchRhs);
+        build_batch_level(B, l, last, rows_cta, out, true);
     }
 }
 
@@ -286,16 +388,32 @@ void batch_apply_layout(gemslr_batch_ctx *B, const double *in, double *out, cuda
         v.live = live;
         return v;
     };
+    auto sweep = [&](int l, int mode, const double *src, double *dst) {
+        const BLevelHost &h = B->lev[l];
+        if (!h.streamed) {
+            launch_btrsv(lv(l), mode, h.rpc, h.smem_bytes, src, B->work, dst, B->scratch, st);
+            return;
+        }
+        // the groups touch different blocks; one after another, each would end in a
+        // wave of its own
+        const int ns = std::min<int>((int)h.units.size(), kBatchStreams);
+        if (ns > 1) GEMSLR_CUDA(cudaEventRecord(B->ev_fork, st));
+        for (int i = 1; i < ns; ++i) GEMSLR_CUDA(cudaStreamWaitEvent(B->side[i - 1], B->ev_fork, 0));
+        for (size_t i = 0; i < h.units.size(); ++i)
+            launch_bstream(lv(l), h.units[i], mode, src, B->work, dst, i % ns == 0 ? st : B->side[i % ns - 1]);
+        for (int i = 1; i < ns; ++i) {
+            GEMSLR_CUDA(cudaEventRecord(B->ev_join[i - 1], B->side[i - 1]));
+            GEMSLR_CUDA(cudaStreamWaitEvent(st, B->ev_join[i - 1], 0));
+        }
+    };
     for (int l = 0; l < ns; ++l) {
         const double *src = l == 0 ? in : nullptr;
-        launch_btrsv(lv(l), 0, B->lev[l].rpc, B->lev[l].smem_bytes, src, B->work, nullptr, B->scratch, st);
+        sweep(l, 0, src, nullptr);
         launch_bcouple(lv(l), src, B->work, st);
         launch_blowrank(lv(l), B->work, st);
     }
-    const BLevelHost &la = B->lev[ns];
-    launch_btrsv(lv(ns), 0, la.rpc, la.smem_bytes, ns == 0 ? in : nullptr, B->work, out, B->scratch, st);
-    for (int l = ns - 1; l >= 0; --l)
-        launch_btrsv(lv(l), 1, B->lev[l].rpc, B->lev[l].smem_bytes, nullptr, B->work, out, B->scratch, st);
+    sweep(ns, 0, ns == 0 ? in : nullptr, out);
+    for (int l = ns - 1; l >= 0; --l) sweep(l, 1, nullptr, out);
 }
 
 void build_segments(gemslr_batch_ctx *B, int rows) {
@@ -559,6 +677,9 @@ gemslr_status setup_batch(int32_t nsys, const gemslr_csr *A, const gemslr_partit
         B->err = (int32_t *)a.alloc(16);
         GEMSLR_CUDA(cudaMemset(B->err, 0, 16));
         set_btrsv_smem_limit(dev_smem_optin());
+        for (cudaStream_t &t : B->side) GEMSLR_CUDA(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
+        GEMSLR_CUDA(cudaEventCreateWithFlags(&B->ev_fork, cudaEventDisableTiming));
+        for (cudaEvent_t &e : B->ev_join) GEMSLR_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         // batch-wide A (block diagonal), permutation maps
         std::vector<int64_t> rp{0}, perm_g(B->N), nsz(nsys), usr_off(nsys + 1, 0);
         std::vector<int32_t> ci, sys_of(B->N);
@@ -604,12 +725,12 @@ gemslr_status setup_batch(int32_t nsys, const gemslr_csr *A, const gemslr_partit
         double best = 1e30;
         int best_rows = B->rows_couple;
         for (int rows : {64, 128, 256}) {
-            for (int l = 0; l + 1 < B->nlev; ++l) build_batch_level(B.get(), l, false, rows, B->lev[l]);
+            for (int l = 0; l + 1 < B->nlev; ++l) build_batch_level(B.get(), l, false, rows, B->lev[l], true);
             const double t = time_ms(B->cap, [&] { batch_apply_layout(B.get(), B->vin, B->zout, B->cap); });
-            if (t < best) { best = t; best_rows = rows; }
+            if (t < 0.98 * best) { best = t; best_rows = rows; }   // differences within the timing noise decide nothing
         }
         B->rows_couple = best_rows;
-        for (int l = 0; l + 1 < B->nlev; ++l) build_batch_level(B.get(), l, false, best_rows, B->lev[l]);
+        for (int l = 0; l + 1 < B->nlev; ++l) build_batch_level(B.get(), l, false, best_rows, B->lev[l], true);
         // the Krylov kernels' rows per CTA is not tuned on a proxy: a norm
         // (one column) prefers long CTAs, while the Gram-Schmidt passes over
         // tens of basis columns are bound by load latency and want many CTAs

@@ -19,6 +19,20 @@ constexpr int kBatchMaxRank = 64;              // k_eff per system in the batche
 constexpr int kBatchThreads = 256;
 constexpr int kKrylovRows = 512;               // batch rows per CTA of the batched Krylov kernels
 
+// Streamed substitutions (blocks whose vectors fit in shared memory for
+// kBatchRhs or half as many right-hand sides, rows of at most 16 entries): work
+// units, one CTA each, grouped by how many fit on an SM.
+constexpr int kBatchSets = 4;                  // sets of warps that take a block's slices in turn
+constexpr int kBatchSliceRows = 32;
+constexpr int kBatchItemBytes = 4096;          // slices of a set are joined into items of about this size
+constexpr int kBatchDepth = 2;                 // ring slots per set
+constexpr int kBatchStreams = 4;               // launches of a level's groups of units side by side
+struct BatchUnits {
+    int32_t n = 0, rpc = 0;    // CTAs; right-hand sides of each (kBatchRhs or kBatchRhs / 2)
+    size_t smem = 0;
+    const int32_t *blk = nullptr, *rhs0 = nullptr;
+};
+
 // One stage level of the batch: the level-l blocks of every system.
 struct BatchLevel {
     int32_t nblk;
@@ -31,7 +45,14 @@ struct BatchLevel {
     const int64_t *blk_r0;     // first batch row of every block
     const int32_t *blk_nr;     // rows of every block
     const int64_t *blk_f0;     // first row of the block in the level's F
-    ChunkView C;               // L and U chunks of every block (lane-per-row layout)
+    ChunkView C;               // L and U chunks of every block (levels that are not streamed)
+    // L and U of every block as slices (streamed levels, kernels.cuh's items): header
+    // int32 {rows - 1, distance to the next slice of the item, 0, flags as in FP64};
+    // {row, d}[rows], padded to 16 bytes; row_bytes(np) per row: pairs of entries.
+    // Rows and columns as (index + 1) * 16: place 0 is a row of zeros, for absent entries
+    StreamView S;
+    const int32_t *F_rows;     // block-local rows with F entries
+    const int32_t *F_blk;      // nblk + 1 ranges of every block's rows in F_rows
     const int64_t *F_rp;       // level rows of all systems, in block order
     const int32_t *F_ci;       // batch row
     const float *F_v;

@@ -2,9 +2,11 @@
 // sides each, one launch per stage of M^{-1} (Alg. 2) over every system, and
 // FGMRES (Sec. 4.1) run for every (system, rhs) pair in lock step.
 // Preconditioner in FP32 (W in BF16, FP32 accumulation), Krylov in FP64.
+#include <type_traits>
+
 #include "batch.cuh"
 #include "device.h"
-#include "ptx.cuh"
+#include "stream.cuh"
 
 namespace gemslr {
 
@@ -142,6 +144,207 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
         const bool keep = MODE == 0 ? SMEM : !(lv.final_up && out_final);
         if (keep) mine[g] = y;
         if (out_final) out_final[r0 * R8 + g] = (double)y;
+    }
+}
+
+// ---- streamed substitutions -------------------------------------------------------------
+// The substitutions of one block for RPC right-hand sides, the vector in shared
+// memory.  Bound by the chain of wavefronts (a 48^3 system's first-level block:
+// about 640 of 20 to 60 rows), so, as in the single-system kernels, a set of warps
+// has its next rows in registers when their wavefront is due, two sets take the
+// slices in turn, a barrier ends every wavefront, and nothing on the chain
+// branches.  A lane holds four right-hand sides of one row: an entry costs it
+// one 16-byte gather and four FMAs.  MODE as in k_btrsv; the rows' sums too (even
+// entries in a0, odd ones in a1, x d + (a0 + a1)).
+// Measured on 96 systems (sides 16 to 48) x 8 right-hand sides: one application
+// 2.67 -> 1.91 ms, the FGMRES solve 152 -> 128 ms; 24 systems (sides 6 to 16) x 3:
+// 0.46 -> 0.18 ms (before: k_btrsv, 16 warps per chunk of one wavefront).
+struct Rhs4 {
+    float v[4];
+};
+__device__ __forceinline__ Rhs4 load4(uint32_t a) {
+    Rhs4 r;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]) : "r"(a) : "memory");
+    return r;
+}
+__device__ __forceinline__ void store4(uint32_t a, const Rhs4 &r) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(r.v[0]), "f"(r.v[1]), "f"(r.v[2]), "f"(r.v[3])
+                 : "memory");
+}
+
+// A row in registers: where its values are, d, and NP pairs of entries.
+template <int NP>
+struct BatchRow {
+    uint32_t at;
+    float d;
+    int4 e[NP];
+};
+// vec: shared address of the vector (its row of zeros) plus the lane's part of a row.
+template <int NP, int RPC>
+__device__ __forceinline__ void fetch_row(uint32_t p, int last, int t, uint32_t vec, BatchRow<NP> &R) {
+    t = min(t, last);
+    constexpr int kUp = RPC / 4;                // 16-byte places to rows of RPC values
+    const int2 ri = lds<int2>(p + kItemHeader + 8 * t);
+    const uint32_t q = p + kItemHeader + ((8 * last + 23) & ~15) + row_bytes(NP) * t;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        const int4 e = lds<int4>(q + 16 * i);
+        R.e[i] = make_int4((int)(vec + kUp * e.x), e.y, (int)(vec + kUp * e.z), e.w);
+    }
+    R.at = vec + kUp * ri.x;
+    R.d = __int_as_float(ri.y);
+}
+
+__device__ __forceinline__ void sets_barrier(int on, int threads) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %0, 0;\n\t@p bar.sync 2, %1;\n\t}" ::"r"(on), "r"(threads) : "memory");
+}
+
+template <int NP, int RPC>
+__device__ __forceinline__ void batch_slices(uint32_t p, uint32_t vec, int slot, int nthreads, int &nsync) {
+    BatchRow<NP> A, B;
+    int4 h = lds<int4>(p);
+    fetch_row<NP, RPC>(p, h.x, slot, vec, A);
+    auto step = [&](const BatchRow<NP> &R, BatchRow<NP> &next) {
+        const int before = h.w >> 24, after = h.w & kSync;
+        const bool mine = slot <= h.x;
+        const uint32_t pn = p + h.y;
+        const int4 hn = lds<int4>(pn);
+#pragma unroll
+        for (int k = 0; k < kBatchSets - 1; ++k) sets_barrier(before > k, nthreads);
+        nsync -= before + after;
+        Rhs4 x[2 * NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            x[2 * i] = load4((uint32_t)R.e[i].x);
+            x[2 * i + 1] = load4((uint32_t)R.e[i].z);
+        }
+        const Rhs4 self = load4(R.at);
+        Rhs4 y;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                a0 = __fmaf_rn(__int_as_float(R.e[i].y), x[2 * i].v[r], a0);
+                a1 = __fmaf_rn(__int_as_float(R.e[i].w), x[2 * i + 1].v[r], a1);
+            }
+            y.v[r] = __fmaf_rn(self.v[r], R.d, __fadd_rn(a0, a1));
+        }
+        if (mine) store4(R.at, y);
+        const bool more = h.y != 0;
+        p = pn;
+        h = hn;
+        sets_barrier(after, nthreads);
+        fetch_row<NP, RPC>(p, h.x, slot, vec, next);    // while the other sets work on the next wavefront
+        return more;
+    };
+    while (step(A, B) && step(B, A)) {
+    }
+}
+
+constexpr int kBatchStreamWarps = 8;            // compute warps of a unit (four walk the stream when RPC is 4)
+
+template <int MODE, int RPC, int NP>
+__global__ void __launch_bounds__(32 * (kBatchStreamWarps + 1))
+k_bstream(const BatchLevel lv, const int32_t *__restrict__ unit_blk, const int32_t *__restrict__ unit_rhs0,
+          const double *__restrict__ in, float *__restrict__ work, double *__restrict__ out_final) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    StreamHead *H = reinterpret_cast<StreamHead *>(smem);
+    constexpr int kSetWarps = RPC / 4;          // 32 rows of RPC / 4 lanes
+    constexpr int kWalk = kBatchSets * kSetWarps, NC = 32 * kBatchStreamWarps, Q = RPC / 4;
+    const int b = unit_blk[blockIdx.x], rhs0 = unit_rhs0[blockIdx.x];
+    if (lv.live && !lv.live[lv.blk_sys[b]]) return;          // the whole CTA
+    const int64_t r0 = lv.blk_r0[b];
+    const int nr = lv.blk_nr[b];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *xs = reinterpret_cast<float *>(smem + sizeof(StreamHead));         // row 0: zeros
+    unsigned char *ring = smem + sizeof(StreamHead) + (size_t)(nr + 1) * RPC * sizeof(float);
+    const int i0 = lv.S.blk_item[b], i1 = lv.S.blk_item[b + 1];
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < lv.S.slots; ++s) {
+            mbar_init(&H->full[s], 1);
+            mbar_init(&H->empty[s], kSetWarps);
+        }
+        H->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if (warp == kBatchStreamWarps) {            // producer
+        produce_items(lv.S, i0, i1, H, ring, lv.err, lane);
+        return;
+    }
+    const int ct = threadIdx.x;
+    float *mine = work + r0 * R8 + rhs0;
+    float4 *x4 = reinterpret_cast<float4 *>(xs);
+    if (ct < Q) x4[ct] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (MODE == 1) {
+        for (int i = ct; i < nr * Q; i += NC) x4[Q + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        compute_barrier<NC>();
+        const int64_t f0 = lv.blk_f0[b];
+        const int fa = lv.F_blk[b], nf = lv.F_blk[b + 1] - fa;
+        for (int t = ct; t < nf * Q; t += NC) {
+            const int i = lv.F_rows[fa + t / Q], part = 4 * (t % Q);
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int64_t p = lv.F_rp[f0 + i]; p < lv.F_rp[f0 + i + 1]; ++p) {
+                const float v = lv.F_v[p];
+                const float4 w = *reinterpret_cast<const float4 *>(work + (int64_t)lv.F_ci[p] * R8 + rhs0 + part);
+                a.x = __fmaf_rn(v, w.x, a.x);
+                a.y = __fmaf_rn(v, w.y, a.y);
+                a.z = __fmaf_rn(v, w.z, a.z);
+                a.w = __fmaf_rn(v, w.w, a.w);
+            }
+            x4[(i + 1) * Q + t % Q] = a;
+        }
+    } else if (in) {
+#pragma unroll 4
+        for (int t = ct; t < nr * Q; t += NC) {
+            const double2 *src = reinterpret_cast<const double2 *>(in + (r0 + t / Q) * R8 + rhs0 + 4 * (t % Q));
+            const double2 u = src[0], v = src[1];
+            x4[Q + t] = make_float4((float)u.x, (float)u.y, (float)v.x, (float)v.y);
+        }
+    } else {
+#pragma unroll 4
+        for (int t = ct; t < nr * Q; t += NC)
+            x4[Q + t] = *reinterpret_cast<const float4 *>(mine + (int64_t)(t / Q) * R8 + 4 * (t % Q));
+    }
+    compute_barrier<NC>();
+    if (warp < kWalk) {
+        const int set = warp / kSetWarps;
+        ItemWalk W(lv.S, H, ring, set);
+        const int lt = 32 * (warp % kSetWarps) + lane;
+        const uint32_t vec = smem_u32(xs) + 16 * (lt % Q);
+        int nsync = lv.S.split[b];
+        for (int g = set; g < i1 - i0; g += kBatchSets) {
+            const uint32_t p = W.item();
+            if (!p) break;
+            batch_slices<NP, RPC>(p, vec, lt / Q, 32 * kWalk, nsync);
+            W.next(lane);
+        }
+        for (; nsync > 0; --nsync) sets_barrier(1, 32 * kWalk);
+    }
+    compute_barrier<NC>();
+    if (*(volatile int *)&H->abort_flag) {
+        if (ct == 0) atomicExch(lv.err, 1);
+        return;
+    }
+    // down: z1; up: the lower levels' up sweeps gather this level's result from
+    // work, nothing reads the first level's
+    const bool keep = MODE == 0 || !(lv.final_up && out_final);
+#pragma unroll 2
+    for (int t = ct; t < nr * Q; t += NC) {
+        float4 y = x4[Q + t];
+        float4 *w = reinterpret_cast<float4 *>(mine + (int64_t)(t / Q) * R8 + 4 * (t % Q));
+        if (MODE == 1) {
+            const float4 z = *w;
+            y = make_float4(z.x - y.x, z.y - y.y, z.z - y.z, z.w - y.w);
+        }
+        if (keep) *w = y;
+        if (out_final) {
+            double2 *o = reinterpret_cast<double2 *>(out_final + (r0 + t / Q) * R8 + rhs0 + 4 * (t % Q));
+            o[0] = make_double2((double)y.x, (double)y.y);
+            o[1] = make_double2((double)y.z, (double)y.w);
+        }
     }
 }
 
@@ -821,12 +1024,48 @@ void launch_btrsv(const BatchLevel &lv, int mode, int rpc, size_t smem_bytes, co
     else launch_btrsv_mode<1>(lv, rpc, smem_bytes, in, work, out_final, scratch, st);
     count_launch();
 }
+template <typename Fn>
+static void with_bstream(int mode, int rpc, int np, Fn f) {
+    auto pick = [&](auto m, auto r) {
+        constexpr int M = decltype(m)::value, R = decltype(r)::value;
+        switch (np) {
+            case 1: return f(k_bstream<M, R, 1>);
+            case 3: return f(k_bstream<M, R, 3>);
+            case 5: return f(k_bstream<M, R, 5>);
+            default: return f(k_bstream<M, R, 8>);
+        }
+    };
+    constexpr std::integral_constant<int, 0> m0;
+    constexpr std::integral_constant<int, 1> m1;
+    constexpr std::integral_constant<int, 4> r4;
+    constexpr std::integral_constant<int, 8> r8;
+    if (mode == 0) rpc == 8 ? pick(m0, r8) : pick(m0, r4);
+    else rpc == 8 ? pick(m1, r8) : pick(m1, r4);
+}
+// shared memory of a unit: rows (and the row of zeros) of rpc right-hand sides, and the ring
+size_t bstream_smem(int64_t rows, int rpc, const StreamView &S) {
+    return sizeof(StreamHead) + (size_t)(rows + 1) * rpc * sizeof(float) + (size_t)S.slots * S.slot_bytes;
+}
+void launch_bstream(const BatchLevel &lv, const BatchUnits &u, int mode, const double *in, float *work, double *out_final,
+                    cudaStream_t st) {
+    if (u.n == 0) return;
+    with_bstream(mode, u.rpc, lv.S.np, [&](auto kernel) {
+        kernel<<<u.n, 32 * (kBatchStreamWarps + 1), u.smem, st>>>(lv, u.blk, u.rhs0, in, work, out_final);
+    });
+    count_launch();
+}
 template <int RPC>
 static void set_btrsv_attr(int bytes) {
     cudaFuncSetAttribute(k_btrsv<0, true, RPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(k_btrsv<1, true, RPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 void set_btrsv_smem_limit(int bytes) {
+    for (int np : {1, 3, 5, 8})
+        for (int mode : {0, 1})
+            for (int rpc : {4, 8})
+                with_bstream(mode, rpc, np, [&](auto kernel) {
+                    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+                });
     set_btrsv_attr<8>(bytes);
     set_btrsv_attr<4>(bytes);
     set_btrsv_attr<2>(bytes);

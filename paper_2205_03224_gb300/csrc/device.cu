@@ -478,8 +478,8 @@ void append_scaling(const Csr &U, int64_t r0, int64_t nr, LaneSlices &out) {
 }
 
 // Slices to items: consecutive rounds of one slice per consumer are joined while
-// every consumer's share keeps its class and stays within kLaneItemBytes.  Returns the slices with kSync.
-int32_t pack_lanes(LaneSlices &s, StreamHost &out) {
+// every consumer's share keeps its class and stays within item_bytes.  Returns the slices with kSync.
+int32_t pack_lanes(LaneSlices &s, size_t item_bytes, StreamHost &out) {
     const size_t nc = out.consumers, ns = s.off.size() - 1;
     auto header = [&](size_t k) { return reinterpret_cast<int32_t *>(s.data.data() + s.off[k]); };
     auto bytes = [&](size_t k) { return s.off[k + 1] - s.off[k]; };
@@ -498,7 +498,7 @@ int32_t pack_lanes(LaneSlices &s, StreamHost &out) {
             bool fits = true;
             for (size_t c = 0; c < nc && k1 + c < ns; ++c)
                 fits = fits && (k1 == k0 || (cls(k1 + c) == cls(k0 + c) && cls(k0 + c) != kLaneScale &&
-                                             share[c] + bytes(k1 + c) <= (size_t)kLaneItemBytes));
+                                             share[c] + bytes(k1 + c) <= item_bytes));
             if (!fits) break;
             for (size_t c = 0; c < nc && k1 + c < ns; ++c) share[c] += bytes(k1 + c);
             k1 = std::min(ns, k1 + nc);
@@ -516,6 +516,24 @@ int32_t pack_lanes(LaneSlices &s, StreamHost &out) {
     return nsync;
 }
 
+// Slices of one factor in the batched layout (batch.cuh).
+void append_batch_rows(const Csr &T, int64_t r0, const Waves &W, bool upper, int np, int max_rows, LaneSlices &out) {
+    auto place = [&](int64_t i) { return (int32_t)((i - r0 + 1) * 16); };
+    for (const SliceRows &s : cut_slices<float>(W, r0, upper, max_rows)) {
+        unsigned char *p = out.add(kItemHeader + pad16((size_t)(8 * s.n)) + (size_t)(row_bytes(np) * s.n), s.n, 0,
+                                   s.sync ? kSync : 0);
+        EntryF32 *head = reinterpret_cast<EntryF32 *>(p);
+        unsigned char *recs = p + pad16((size_t)(8 * s.n));
+        for (int64_t t = 0; t < s.n; ++t) {
+            const int64_t i = s.rows[t], pdiag = upper ? diagonal(T, i) : -1;
+            head[t] = {place(i), upper ? inv_entry<float>(T, pdiag) : 1.f};
+            EntryF32 *rec = reinterpret_cast<EntryF32 *>(recs + row_bytes(np) * t);
+            for (int64_t q = T.rp[i]; q < T.rp[i + 1]; ++q)
+                if (T.ci[q] != i) *rec++ = {place(T.ci[q]), stored_entry<float>(T, q, pdiag)};
+        }
+    }
+}
+
 }  // namespace
 
 void build_chunks(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, ChunkHost &out, int max_rows) {
@@ -526,7 +544,22 @@ void build_chunks(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, Ch
         append_factor_chunks(U, bp[b], bp[b + 1], true, out, max_rows);
         out.blk_chunk.push_back((int32_t)(out.off.size() - 1));
     }
-    if (out.data.empty()) out.data.resize(16, 0);
+}
+
+void append_batch_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, int max_rows, size_t item_bytes,
+                         StreamHost &out, int64_t &l_bytes, int64_t &u_bytes) {
+    validate_tri(L, bp, false);
+    validate_tri(U, bp, true);
+    for (size_t b = 0; b + 1 < bp.size(); ++b) {
+        LaneSlices s;
+        append_batch_rows(L, bp[b], order_rows(L, bp[b], bp[b + 1], false), false, out.np, max_rows, s);
+        const size_t lower = s.data.size();
+        append_batch_rows(U, bp[b], order_rows(U, bp[b], bp[b + 1], true), true, out.np, max_rows, s);
+        l_bytes += (int64_t)lower;
+        u_bytes += (int64_t)(s.data.size() - lower);
+        out.split.push_back(pack_lanes(s, item_bytes, out));
+        out.blk_item.push_back((int32_t)(out.off.size() - 1));
+    }
 }
 
 template <typename VT>
@@ -562,7 +595,7 @@ void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, St
             append_lanes<VT>(L, r0, wl[b], false, out.np, s);
             append_scaling<VT>(U, r0, bp[b + 1] - r0, s);
             append_lanes<VT>(U, r0, wu[b], true, out.np, s);
-            out.split.push_back(pack_lanes(s, out));
+            out.split.push_back(pack_lanes(s, kLaneItemBytes, out));
         }
         out.blk_item.push_back((int32_t)(out.off.size() - 1));
         wl[b] = Waves();

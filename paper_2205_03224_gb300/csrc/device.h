@@ -138,6 +138,11 @@ struct StreamHost {                    // single-system substitutions (see Strea
     int slot_bytes = 0;                // largest item
     int maxwf_L = 0, maxwf_U = 0;      // wavefronts (largest over the blocks)
 };
+// batched streamed substitutions (batch.cuh), appended block by block to `out`
+// (np, consumers set): slices of max_rows rows, in items of about item_bytes;
+// their bytes are added to l_bytes and u_bytes
+void append_batch_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, int max_rows, size_t item_bytes,
+                         StreamHost &out, int64_t &l_bytes, int64_t &u_bytes);
 template <typename VT>
 void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, StreamHost &out);
 
