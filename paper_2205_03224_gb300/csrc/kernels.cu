@@ -45,6 +45,23 @@ k_couple(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restr
     const int64_t i0 = (int64_t)blockIdx.x * kCoupleRows;
     const int64_t i1 = min(i0 + (int64_t)kCoupleRows, lv.stail);
     const int64_t i = i0 + threadIdx.x;
+    const int k = lv.k, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    // absent rows, columns and partials are left out for real values; complex sums
+    // keep them (zeros), so that their products are contracted as they always were
+    constexpr bool kSkip = !std::is_same_v<VT, zc>;
+    const int nr = (int)(i1 - i0), nq = kSkip ? (nr + 31) >> 5 : 8;   // rows per lane of the W^T z part
+    static_assert(kCoupleRows == 256, "eight rows per lane");
+    // this warp's columns of W for its first pass, before anything waits for memory
+    WT wv[4][8];
+    auto load_w = [&](int cb) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const WT *wc = lv.W + (int64_t)min(cb + u * nwarp, k - 1) * lv.stail + i0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) wv[u][q] = wc[min(lane + 32 * q, nr - 1)];
+        }
+    };
+    if (warp < k) load_w(warp);
     VT z = 0;
     if (i < i1) {
         z = in ? (VT)in[lv.e + i] : work[lv.e + i];
@@ -67,64 +84,63 @@ k_couple(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restr
         work[lv.e + i] = z;
     }
     zs[threadIdx.x] = z;
-    const int k = lv.k;
     if (k == 0) return;
     __syncthreads();
     // partial W^T z2: warp w takes columns w, w+nw, w+2nw, w+3nw together, each
-    // lane its eight rows of every one of them, all 32 loads before any FMA
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const int64_t nr = i1 - i0;
-    static_assert(kCoupleRows == 256, "eight rows per lane");
+    // lane its rows (up to eight) of every one of them, all loads before any FMA.
+    // A single CTA's partials are the sums themselves.
+    const bool only = kSkip && gridDim.x == 1;
     for (int cb = warp; cb < k; cb += 4 * nwarp) {
-        WT wv[4][8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int c = min(cb + u * nwarp, k - 1);
-            const WT *wc = lv.W + (int64_t)c * lv.stail + i0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) wv[u][q] = wc[min((int64_t)(lane + 32 * q), nr - 1)];
-        }
+        if (cb != warp) load_w(cb);
         VT acc[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             acc[u] = 0;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) acc[u] += wval_h<VT, WT>(wv[u][q]) * zs[lane + 32 * q];   // zs = 0 past i1
+            for (int q = 0; q < 8; ++q)
+                if (q < nq) acc[u] += wval_h<VT, WT>(wv[u][q]) * zs[lane + 32 * q];   // zs = 0 past i1
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int c = cb + u * nwarp;        // uniform over the warp
             if (c < k) {
-                const VT t = warp_sum(acc[u]);
-                if (lane == 0) partial[(int64_t)c * gridDim.x + blockIdx.x] = t;
+                const VT t = warp_sum_of(acc[u], kSkip ? nr : 32);
+                if (lane == 0) {
+                    if (only) ts[c] = t;
+                    else partial[(int64_t)c * gridDim.x + blockIdx.x] = t;
+                }
             }
         }
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
     // u = H t: every thread's row of H is loaded while the partials are reduced
     constexpr int kHPre = sizeof(VT) == 4 ? 32 : 16;
     VT hrow[kHPre];
     const int c = threadIdx.x;
+    if (!only) {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = (atomicAdd(counter, 1u) == gridDim.x - 1);
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+    }
 #pragma unroll
     for (int d = 0; d < kHPre; ++d) hrow[d] = (c < k && d < k) ? lv.H[c + (int64_t)d * k] : (VT)0;
-    reduce_columns<VT>(partial, (int)gridDim.x, k, ts);
+    if (only) __syncthreads();
+    else reduce_columns<VT>(partial, (int)gridDim.x, k, ts);
     for (int cc2 = c; cc2 < k; cc2 += blockDim.x) {
         VT acc = 0;
         if (cc2 == c) {
 #pragma unroll
-            for (int d = 0; d < kHPre; ++d) acc += hrow[d] * (d < k ? ts[d] : (VT)0);
+            for (int d = 0; d < kHPre; ++d)
+                if (!kSkip || d < k) acc += hrow[d] * (d < k ? ts[d] : (VT)0);
             for (int d = kHPre; d < k; ++d) acc += lv.H[cc2 + (int64_t)d * k] * ts[d];
         } else {
             for (int d = 0; d < k; ++d) acc += lv.H[cc2 + (int64_t)d * k] * ts[d];
         }
         u_out[cc2] = acc;
     }
-    if (threadIdx.x == 0) *counter = 0u;
+    if (threadIdx.x == 0 && !only) *counter = 0u;
 }
 
 // ---- bounded-wait self-test ---------------------------------------------------

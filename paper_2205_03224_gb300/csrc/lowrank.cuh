@@ -20,7 +20,7 @@ template <> __device__ __forceinline__ zc wval_h<zc, zc>(zc w) { return conj(w);
 
 // Row g's share of the previous level's W u (see PendingLowRank): sixteen
 // columns at a time with all their loads issued first (columns past k load
-// the last column again and are multiplied by zero).  u is read through L2:
+// the last column again and are not added).  u is read through L2:
 // the coupling kernel that reads it also rewrites it in its finisher.
 template <typename VT, typename WT>
 __device__ __forceinline__ VT pending_row(const PendingLowRank<VT, WT> &pl, int64_t g) {
@@ -35,10 +35,19 @@ __device__ __forceinline__ VT pending_row(const PendingLowRank<VT, WT> &pl, int6
             wv[q] = w[(int64_t)c * pl.ld];
             uv[q] = c0 + q < pl.k ? ldcg(pl.u + c) : (VT)0;
         }
+        const int left = std::is_same_v<VT, zc> ? 16 : pl.k - c0;   // complex: contracted as always
+        if (left >= 16) {
 #pragma unroll
-        for (int q = 0; q < 16; q += 2) {
-            a0 += wval<VT, WT>(wv[q]) * uv[q];
-            a1 += wval<VT, WT>(wv[q + 1]) * uv[q + 1];
+            for (int q = 0; q < 16; q += 2) {
+                a0 += wval<VT, WT>(wv[q]) * uv[q];
+                a1 += wval<VT, WT>(wv[q + 1]) * uv[q + 1];
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 16; q += 2) {
+                if (q < left) a0 += wval<VT, WT>(wv[q]) * uv[q];
+                if (q + 1 < left) a1 += wval<VT, WT>(wv[q + 1]) * uv[q + 1];
+            }
         }
     }
     return a0 + a1;

@@ -21,15 +21,26 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 
 
+// Sum over the first `live` lanes (the others hold zeros), in the order of
+// warp_sum without the stages that would add zeros: an FP64 addition holds its SM
+// quarter for 64 cycles.  Valid in lane 0; live is uniform.
+template <typename T>
+__device__ __forceinline__ T warp_sum_of(T v, int live) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (live > o) v += shfl_xor(v, o);
+    return v;
+}
+
 // Column sums of per-CTA partials (column-major: partial c of CTA p at
 // c * nparts + p, so a warp's loads of one column are contiguous) into
 // out[0..ncols1) (shared memory), by all warps of the finishing CTA.  Warp w
 // takes columns w, w+nw, w+2nw, w+3nw together; its lanes load up to eight
 // partials each for all four columns before any addition (one memory round
 // trip per pass of 256 CTAs), add them in a fixed pairwise tree and finish
-// with a warp reduction.  The summation order is fixed (deterministic).  Short dependent
-// chains matter here: one FP64 add takes on the order of a hundred cycles on
-// this part when nothing else is in flight.
+// with a warp reduction.  The summation order is fixed (deterministic); additions
+// of absent partials are left out (one FP64 add takes on the order of a hundred
+// cycles on this part when nothing else is in flight).
 template <typename T>
 __device__ void reduce_columns(const T *partial, int nparts, int ncols1, T *out) {
     constexpr int RP = 8, CW = 4;
@@ -49,15 +60,26 @@ __device__ void reduce_columns(const T *partial, int nparts, int ncols1, T *out)
                     v[u][q] = (c < ncols1 && p < nparts) ? ldcg(partial + (int64_t)c * nparts + p) : (T)0;
                 }
             }
+            if (nparts <= 32) {
 #pragma unroll
-            for (int u = 0; u < CW; ++u)
-                acc[u] += ((v[u][0] + v[u][1]) + (v[u][2] + v[u][3])) + ((v[u][4] + v[u][5]) + (v[u][6] + v[u][7]));
+                for (int u = 0; u < CW; ++u) acc[u] = v[u][0];
+            } else if (nparts <= 64) {
+#pragma unroll
+                for (int u = 0; u < CW; ++u) acc[u] = v[u][0] + v[u][1];
+            } else if (nparts <= 128) {
+#pragma unroll
+                for (int u = 0; u < CW; ++u) acc[u] = (v[u][0] + v[u][1]) + (v[u][2] + v[u][3]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < CW; ++u)
+                    acc[u] += ((v[u][0] + v[u][1]) + (v[u][2] + v[u][3])) + ((v[u][4] + v[u][5]) + (v[u][6] + v[u][7]));
+            }
         }
 #pragma unroll
         for (int u = 0; u < CW; ++u) {
             const int c = cb + u * nw;          // uniform over the warp
             if (c < ncols1) {
-                const T t = warp_sum(acc[u]);
+                const T t = warp_sum_of(acc[u], nparts);
                 if (lane == 0) out[c] = t;
             }
         }
