@@ -21,7 +21,12 @@ namespace gemslr {
 
 namespace {
 
-constexpr int kZTile = 1024;           // rows per tile of the V^H w reduction
+// Rows per tile of the V^H w reduction.  The set-up's Arnoldi keeps 1024 (the order
+// of its sums decides the bits of W and H).  FGMRES takes 256: the products are
+// bound by the FP64 pipe (an instruction holds an SM quarter for 64 cycles), and
+// at 32^3 1024 rows give 32 CTAs for 152 SMs.  With the tail below and k_zsub's
+// batched loads, 57 iterations at 32^3: 83.2 -> 78.6 ms.
+constexpr int kZTile = 1024, kZSolveTile = 256;
 constexpr int kZThreads = 256;
 
 // Per-step results of the Hessenberg kernel (device; read by the host).
@@ -73,24 +78,33 @@ __global__ void __launch_bounds__(256) k_zspmv(int64_t n, const int64_t *__restr
 // stages tiles of w in shared memory; warp q takes the columns c = q mod 8 (and
 // the norm slot) over the tile; per-CTA sums go to partials (column-major),
 // and the last CTA reduces them in a fixed order (deterministic).
+template <int TILE>
 __global__ void __launch_bounds__(kZThreads) k_zdots(int64_t len, const zc *__restrict__ V, int64_t ldv, int ncols,
                                                      const zc *__restrict__ w, zc *__restrict__ partial,
                                                      unsigned *__restrict__ counter, zc *__restrict__ out) {
-    __shared__ zc ws[kZTile];
+    __shared__ zc ws[TILE];
     __shared__ zc acc[kMaxCols + 1];
     __shared__ int last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int c = threadIdx.x; c <= ncols; c += blockDim.x) acc[c] = zc(0.0);
-    for (int64_t t0 = (int64_t)blockIdx.x * kZTile; t0 < len; t0 += (int64_t)gridDim.x * kZTile) {
-        const int nr = (int)min((int64_t)kZTile, len - t0);
+    for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < len; t0 += (int64_t)gridDim.x * TILE) {
+        const int nr = (int)min((int64_t)TILE, len - t0);
         __syncthreads();
-        for (int i = threadIdx.x; i < kZTile; i += blockDim.x) ws[i] = i < nr ? w[t0 + i] : zc(0.0);
+        for (int i = threadIdx.x; i < TILE; i += blockDim.x) ws[i] = i < nr ? w[t0 + i] : zc(0.0);
         __syncthreads();
         for (int c = warp; c <= ncols; c += nw) {
             zc s(0.0);
             if (c < ncols) {
                 const zc *vc = V + (int64_t)c * ldv + t0;
-                for (int i = lane; i < nr; i += 32) s += conj(vc[i]) * ws[i];
+                if constexpr (TILE == kZSolveTile) {     // every load of the tile before its arithmetic
+                    zc v[TILE / 32];
+#pragma unroll
+                    for (int q = 0; q < TILE / 32; ++q) v[q] = lane + 32 * q < nr ? vc[lane + 32 * q] : zc(0.0);
+#pragma unroll
+                    for (int q = 0; q < TILE / 32; ++q) s += conj(v[q]) * ws[lane + 32 * q];
+                } else {
+                    for (int i = lane; i < nr; i += 32) s += conj(vc[i]) * ws[i];
+                }
             } else {
                 double q = 0.0;
                 for (int i = lane; i < nr; i += 32) q += abs2(ws[i]);
@@ -121,7 +135,15 @@ __global__ void __launch_bounds__(256) k_zsub(int64_t len, const zc *__restrict_
     __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
         zc a = w[i];
-        for (int c = 0; c < ncols; ++c) a -= V[(int64_t)c * ldv + i] * hs[c];
+        int c0 = 0;
+        for (; c0 + 8 <= ncols; c0 += 8) {      // eight columns' loads in flight together
+            zc v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = V[(int64_t)(c0 + u) * ldv + i];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) a -= v[u] * hs[c0 + u];
+        }
+        for (; c0 < ncols; ++c0) a -= V[(int64_t)c0 * ldv + i] * hs[c0];
         w[i] = a;
     }
 }
@@ -154,39 +176,48 @@ __global__ void k_zcycle_start(int m, const zc *__restrict__ n2, zc *__restrict_
 // breakdown test h_{j+1,j} <= 1e-14 ||A z_j||, the previous rotations, the
 // new complex Givens rotation [[conj(c), conj(s)], [-s, c]] with
 // c = h_jj / d, s = h_{j+1,j} / d, d = sqrt(|h_jj|^2 + h_{j+1,j}^2), and
-// g_{j+1} = -s g_j, g_j = conj(c) g_j.  One thread (the column is short).
-__global__ void k_ztail(int j, int m, zc *__restrict__ H, zc *__restrict__ cs, zc *__restrict__ sn,
-                        zc *__restrict__ g, const zc *__restrict__ h1, const zc *__restrict__ h2,
-                        const zc *__restrict__ nb, ZCtl *__restrict__ ctl) {
-    if (threadIdx.x != 0) return;
-    zc *col = H + (int64_t)j * (m + 1);
-    for (int i = 0; i <= j; ++i) col[i] = h1[i] + h2[i];
-    const double wn0 = sqrt(h1[j + 1].re);
-    const double beta = sqrt(nb->re);
-    col[j + 1] = zc(beta);
-    const bool breakdown = beta <= 1e-14 * wn0;
-    for (int i = 0; i < j; ++i) {
-        const zc t = conj(cs[i]) * col[i] + conj(sn[i]) * col[i + 1];
-        col[i + 1] = -(sn[i] * col[i]) + cs[i] * col[i + 1];
-        col[i] = t;
+// g_{j+1} = -s g_j, g_j = conj(c) g_j.  One warp: the column and the rotations
+// are read together into shared memory and the last rows written back together;
+// one thread runs the chain of rotations, whose carried entry stays in registers.
+__global__ void __launch_bounds__(32)
+k_ztail(int j, int m, zc *__restrict__ H, zc *__restrict__ cs, zc *__restrict__ sn, zc *__restrict__ g,
+        const zc *__restrict__ h1, const zc *__restrict__ h2, const zc *__restrict__ nb, ZCtl *__restrict__ ctl) {
+    __shared__ zc col[kMaxCols + 1], scs[kMaxCols], ssn[kMaxCols];
+    const double wn0 = sqrt(h1[j + 1].re), beta = sqrt(nb->re);
+    const zc gj = g[j];
+    for (int i = threadIdx.x; i <= j; i += 32) {
+        col[i] = h1[i] + h2[i];
+        scs[i] = i < j ? cs[i] : zc(0.0);
+        ssn[i] = i < j ? sn[i] : zc(0.0);
     }
-    const double d = hypot(hypot(col[j].re, col[j].im), beta);
-    zc c(1.0), s(0.0);
-    if (d > 0.0) {
-        c = zc(col[j].re / d, col[j].im / d);
-        s = zc(beta / d);
+    __syncwarp();
+    if (threadIdx.x == 0) {
+        zc carried = col[0];
+        for (int i = 0; i < j; ++i) {
+            const zc next = col[i + 1], c = scs[i], s = ssn[i];
+            col[i] = conj(c) * carried + conj(s) * next;
+            carried = -(s * carried) + c * next;
+        }
+        const double d = hypot(hypot(carried.re, carried.im), beta);
+        zc c(1.0), s(0.0);
+        if (d > 0.0) {
+            c = zc(carried.re / d, carried.im / d);
+            s = zc(beta / d);
+        }
+        cs[j] = c;
+        sn[j] = s;
+        col[j] = zc(d);
+        const zc gn = -(s * gj);
+        g[j + 1] = gn;
+        g[j] = conj(c) * gj;
+        ctl->beta = beta;
+        ctl->breakdown = beta <= 1e-14 * wn0 ? 1 : 0;
+        const double r = hypot(gn.re, gn.im);
+        ctl->resid = r;
+        ctl->nonfinite = (isfinite(r) && isfinite(d)) ? 0 : 1;
     }
-    cs[j] = c;
-    sn[j] = s;
-    col[j] = zc(d);
-    col[j + 1] = zc(0.0);
-    g[j + 1] = -(s * g[j]);
-    g[j] = conj(c) * g[j];
-    ctl->beta = beta;
-    ctl->breakdown = breakdown ? 1 : 0;
-    const double r = hypot(g[j + 1].re, g[j + 1].im);
-    ctl->resid = r;
-    ctl->nonfinite = (isfinite(r) && isfinite(d)) ? 0 : 1;
+    __syncwarp();
+    for (int i = threadIdx.x; i <= j; i += 32) H[(int64_t)j * (m + 1) + i] = col[i];
 }
 
 // y = R^{-1} g[0:jd] for the rotated (upper triangular) Hessenberg matrix.
@@ -254,9 +285,10 @@ namespace {
 
 template <typename T> T *zalloc(ZState &z, size_t count) { return (T *)z.arena->alloc(sizeof(T) * std::max<size_t>(count, 1)); }
 
+template <int TILE = kZTile>
 void zdots(ZState &z, int64_t len, const zc *V, int64_t ldv, int ncols, const zc *w, zc *out, cudaStream_t st) {
-    const int grid = grid_of(len, kZTile, z.red_grid);
-    k_zdots<<<grid, kZThreads, 0, st>>>(len, V, ldv, ncols, w, z.partial, z.counter, out);
+    const int grid = grid_of(len, TILE, z.red_grid);
+    k_zdots<TILE><<<grid, kZThreads, 0, st>>>(len, V, ldv, ncols, w, z.partial, z.counter, out);
     count_launch();
 }
 
@@ -535,7 +567,7 @@ gemslr_status z_solve(ZState *zp, const zc *b, zc *x, const gemslr_solve_opts &o
     k_zgather<<<gs, 256, 0, st>>>(n, z.perm, b, z.bh);
     count_launch();
     zfill(n, z.xh, zc(0.0), z.sms, st);
-    zdots(z, n, nullptr, n, 0, z.bh, z.nb, st);
+    zdots<kZSolveTile>(z, n, nullptr, n, 0, z.bh, z.nb, st);
     const double bnorm = std::sqrt(read_z(z, z.nb, st).real());
     gemslr_status status = GEMSLR_OK;
     if (!std::isfinite(bnorm) || bnorm == 0.0) {
@@ -563,11 +595,11 @@ gemslr_status z_solve(ZState *zp, const zc *b, zc *x, const gemslr_solve_opts &o
             zc *vj = z.V + (size_t)j * n, *zj = z.Z + (size_t)j * n;
             apply_levels<zc, zc>(z.d, 0, vj, zj, nullptr, st);      // z_j = M^{-1} v_j
             zspmv(z, zj, nullptr, z.w, st);                        // w = A z_j
-            zdots(z, n, z.V, n, j + 1, z.w, z.h1, st);            // classical Gram-Schmidt, two passes
+            zdots<kZSolveTile>(z, n, z.V, n, j + 1, z.w, z.h1, st);            // classical Gram-Schmidt, two passes
             zsub(n, z.V, n, j + 1, z.h1, z.w, z.sms, st);
-            zdots(z, n, z.V, n, j + 1, z.w, z.h2, st);
+            zdots<kZSolveTile>(z, n, z.V, n, j + 1, z.w, z.h2, st);
             zsub(n, z.V, n, j + 1, z.h2, z.w, z.sms, st);
-            zdots(z, n, nullptr, n, 0, z.w, z.nb, st);
+            zdots<kZSolveTile>(z, n, nullptr, n, 0, z.w, z.nb, st);
             k_ztail<<<1, 32, 0, st>>>(j, m, z.H, z.cs, z.sn, z.g, z.h1, z.h2, z.nb, z.ctl);
             count_launch();
             zscale(n, z.w, z.nb, z.V + (size_t)(j + 1) * n, z.sms, st);
@@ -584,7 +616,7 @@ gemslr_status z_solve(ZState *zp, const zc *b, zc *x, const gemslr_solve_opts &o
         k_zupdate<<<gs, 256, 0, st>>>(n, z.Z, n, jd, z.y, z.xh);
         count_launch(2);
         zspmv(z, z.xh, z.bh, z.w, st);                              // r = b - A x
-        zdots(z, n, nullptr, n, 0, z.w, z.nb, st);
+        zdots<kZSolveTile>(z, n, nullptr, n, 0, z.w, z.nb, st);
         rnorm = std::sqrt(read_z(z, z.nb, st).real());
         if (!std::isfinite(rnorm)) { nonfinite = true; break; }
         converged = rnorm <= tol;
