@@ -50,7 +50,7 @@ struct gemslr_ctx {
     KrylovCtl *ctl = nullptr;
     KrylovCtl *ctl_host = nullptr;      // pinned
     double *n2_host = nullptr;          // pinned
-    int red_grid = 0;
+    int red_grid = 0, solve_grid = 0;   // CTAs of the reductions: set-up, FGMRES
     double *vin = nullptr, *zout = nullptr;   // fixed in/out of M^{-1} inside the FGMRES step
     int32_t *err_host = nullptr;              // pinned copy of the substitution error word
     double setup_ms = 0.0;
@@ -127,6 +127,10 @@ void ensure_krylov(gemslr_ctx *h, int m) {
         h->r = (double *)h->arena.alloc(8 * n);
         h->w = (double *)h->arena.alloc(8 * n);
         h->red_grid = sm_count();                 // one CTA per SM: few partials for the finisher
+        // FGMRES on small systems: a CTA per 256 rows.  At n = 1,024 the last CTA
+        // reduces 4 partials per column instead of 152 (FP64 additions, 64 cycles
+        // each), and the sums themselves are short: MEASURE
+        h->solve_grid = (int)std::min<int64_t>(h->red_grid, (n + kReduceThreads - 1) / kReduceThreads);
         h->partial = (double *)h->arena.alloc(8 * (size_t)h->red_grid * (2 * kMaxCols + 4));
         h->counter = (unsigned *)h->arena.alloc(16);
         GEMSLR_CUDA(cudaMemset(h->counter, 0, 16));
@@ -444,7 +448,7 @@ void fgmres_step(gemslr_ctx *h, cudaStream_t st) {
     if (h->spmv_lanes <= 8) {       // short rows: the product is fused into the first pass
         ProfScope ps("spmv_gs_dots", st);
         launch_gs_spmv_dots(n, h->A_rp, h->A_ci, h->A_v, h->zout, h->Z, h->V, n, h->w, h->partial, h->counter,
-                            h->ctl, h->Hs, h->cs, h->sn, h->g, h->h2, h->red_grid, st);
+                            h->ctl, h->Hs, h->cs, h->sn, h->g, h->h2, h->solve_grid, st);
     } else {
         {
             ProfScope ps("spmv_A", st);
@@ -452,17 +456,17 @@ void fgmres_step(gemslr_ctx *h, cudaStream_t st) {
         }
         ProfScope ps("gs_dots", st);
         launch_gs_dots(n, h->V, n, h->w, h->partial, h->counter, h->ctl, h->Hs, h->cs, h->sn, h->g, h->h2,
-                       h->red_grid, st);
+                       h->solve_grid, st);
     }
     {
         ProfScope ps("gs_sub", st);
         launch_gs_sub(n, h->V, n, h->w, h->partial, h->counter, h->ctl, h->Hs, h->cs, h->sn, h->g, h->h2,
-                      h->red_grid, st, h->vin);
+                      h->solve_grid, st, h->vin);
     }
     {
         ProfScope ps("gs_sub2", st);
         launch_gs_sub2(n, h->V, n, h->w, h->h2, h->partial, h->counter, h->ctl, h->Hs, h->cs, h->sn, h->g,
-                       h->red_grid, st);
+                       h->solve_grid, st);
         launch_gs_scale(n, h->V, n, h->w, h->ctl, h->vin, st);
     }
 }
@@ -506,7 +510,7 @@ void fgmres_step_d(gemslr_ctx *h, cudaStream_t st) {
     // the SMs the level-0 substitutions leave free (one CTA per SM, none
     // sharing an SM with a substitution CTA); the reduction below needs both
     const int nb0 = h->host.lev.empty() ? 0 : (int)h->host.lev[0].bp.size() - 1;
-    const int fix_grid = std::max(16, h->red_grid - nb0);
+    const int fix_grid = std::min(h->solve_grid, std::max(16, h->red_grid - nb0));
     GEMSLR_CUDA(cudaEventRecord(h->ev_fork, st));
     GEMSLR_CUDA(cudaStreamWaitEvent(h->aux_stream, h->ev_fork, 0));
     {
@@ -519,7 +523,7 @@ void fgmres_step_d(gemslr_ctx *h, cudaStream_t st) {
     {
         ProfScope ps("dgs_spmv_dots", st);
         launch_dgs_dots(n, h->A_rp, h->A_ci, h->A_v, h->zout, h->Z, h->V, n, h->vin, h->w, h->partial, h->counter,
-                        h->ctl, B, h->red_grid, st);
+                        h->ctl, B, h->solve_grid, st);
     }
     // the Hessenberg bookkeeping and the stopping test beside the next direction
     GEMSLR_CUDA(cudaEventRecord(h->ev_fork2, st));
@@ -542,11 +546,11 @@ void fgmres_cycle_end_d(gemslr_ctx *h, cudaStream_t st) {
     const int64_t n = h->host.n;
     const DgsBufs B = dgs_bufs(h);
     launch_dgs_fix(n, h->V, n, h->ctl, B, 0, 8 * h->red_grid, false, st);   // the last step's v_j
-    launch_dgs_close(n, h->V, n, h->vin, h->partial, h->counter, h->ctl, B, h->red_grid, st);
+    launch_dgs_close(n, h->V, n, h->vin, h->partial, h->counter, h->ctl, B, h->solve_grid, st);
     launch_lsq2(h->ctl, h->Hs, h->g, h->Rz, h->y, st);
     launch_update_x(n, h->Z, n, h->ctl, h->y, h->xh, st);
     launch_spmv(n, h->A_rp, h->A_ci, h->A_v, h->xh, h->bh, h->r, h->spmv_lanes, st);
-    launch_norm2(n, h->r, h->partial, h->counter, h->n2 + 1, h->red_grid, st);
+    launch_norm2(n, h->r, h->partial, h->counter, h->n2 + 1, h->solve_grid, st);
 }
 
 // End of a cycle: x += Z y, r = b - A x, ||r||^2 into n2[1].
@@ -555,7 +559,7 @@ void fgmres_cycle_end(gemslr_ctx *h, cudaStream_t st) {
     launch_lsq(h->ctl, h->Hs, h->g, h->y, st);
     launch_update_x(n, h->Z, n, h->ctl, h->y, h->xh, st);
     launch_spmv(n, h->A_rp, h->A_ci, h->A_v, h->xh, h->bh, h->r, h->spmv_lanes, st);
-    launch_norm2(n, h->r, h->partial, h->counter, h->n2 + 1, h->red_grid, st);
+    launch_norm2(n, h->r, h->partial, h->counter, h->n2 + 1, h->solve_grid, st);
 }
 
 // Host-driven loop (used while profiling): the host reads the control block
@@ -1125,7 +1129,7 @@ gemslr_status gemslr_fgmres_solve(gemslr_handle h, const double *b_dev, double *
             gemslr_solve_info &inf = info[c];
             std::memset(&inf, 0, sizeof(inf));
             launch_gather(n, h->perm, b_dev + (size_t)c * n, h->bh, st);
-            launch_norm2(n, h->bh, h->partial, h->counter, h->n2, h->red_grid, st);
+            launch_norm2(n, h->bh, h->partial, h->counter, h->n2, h->solve_grid, st);
             const double bn2 = read_scalar(h, h->n2, st);
             const double bnorm = std::sqrt(bn2);
             if (!std::isfinite(bnorm) || bnorm == 0.0) {

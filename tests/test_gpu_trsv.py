@@ -63,15 +63,9 @@ def _triangles(rng, n, most, band, chain, cplx):
     return out
 
 
-@pytest.mark.parametrize("kind", ["fp64", "mixed", "complex"])
-@pytest.mark.parametrize("name", sorted(CASES))
-def test_substitutions_against_plain_solves(name, kind):
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_03224_gb300 import Gemslr
+def _system(name, cplx):
+    """(random generator, blocks, sizes, matrix, partition, factors) of one case."""
     sizes, most, band, chain = CASES[name]
-    cplx = kind == "complex"
     rng = np.random.default_rng(len(name) + most)
     blocks = [_triangles(rng, n, most, band, chain, cplx) for n in sizes]
     d, tail = sum(sizes), 5
@@ -86,13 +80,53 @@ def test_substitutions_against_plain_solves(name, kind):
     part = dict(perm=np.arange(n, dtype=np.int32), level_ptr=np.array([0, d, n], dtype=np.int64),
                 nblk=np.array([len(sizes), 1], dtype=np.int32),
                 block_ptr=np.concatenate([np.cumsum([0] + sizes), [0, tail]]).astype(np.int64))
-    G = Gemslr.from_factors(A, part, fac, precision="mixed" if kind == "mixed" else "fp64")
-    r = rng.uniform(-1, 1, n) + (1j * rng.uniform(-1, 1, n) if cplx else 0)
-    z = G.apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    return rng, blocks, sizes, A, part, fac
+
+
+def _solved(blocks, sizes, r):
     ref = r.copy()
     o = 0
     for (L, U), m in zip(blocks, sizes):
         ref[o:o + m] = lu_solve(L, U, r[o:o + m])
         o += m
+    return ref
+
+
+@pytest.mark.parametrize("kind", ["fp64", "mixed", "complex"])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_substitutions_against_plain_solves(name, kind):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_03224_gb300 import Gemslr
+    cplx = kind == "complex"
+    rng, blocks, sizes, A, part, fac = _system(name, cplx)
+    G = Gemslr.from_factors(A, part, fac, precision="mixed" if kind == "mixed" else "fp64")
+    r = rng.uniform(-1, 1, A.n) + (1j * rng.uniform(-1, 1, A.n) if cplx else 0)
+    z = G.apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    ref = _solved(blocks, sizes, r)
     tol = 3e-5 if kind == "mixed" else 1e-13
     assert np.max(np.abs(z - ref)) <= tol * np.max(np.abs(ref)), np.max(np.abs(z - ref))
+
+
+# The batched substitutions (FP32): one right-hand side, a partial group and a full
+# one; blocks of one row up to several thousand; systems whose rows are too long
+# for the stored records.
+@pytest.mark.parametrize("nrhs", [1, 5, 8])
+@pytest.mark.parametrize("name", sorted(set(CASES) - {"global_vector"}))
+def test_batched_substitutions_against_plain_solves(name, nrhs):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_03224_gb300 import GemslrBatch
+    sy = [_system(name, False), _system("two_entries", False)]
+    B = GemslrBatch.from_factors([s[3] for s in sy], [s[4] for s in sy], [s[5] for s in sy])
+    rng = np.random.default_rng(nrhs)
+    r = [rng.uniform(-1, 1, (nrhs, s[3].n)) for s in sy]
+    z = B.apply(torch.from_numpy(np.concatenate([a.ravel() for a in r])).cuda(), nrhs).cpu().numpy()
+    o = 0
+    for (_, blocks, sizes, A, _, _), rs in zip(sy, r):
+        for q in range(nrhs):
+            got, ref = z[o:o + A.n], _solved(blocks, sizes, rs[q])
+            o += A.n
+            assert np.max(np.abs(got - ref)) <= 3e-5 * np.max(np.abs(ref)), (q, np.max(np.abs(got - ref)))
