@@ -50,7 +50,7 @@ FP64_PEAK_GFLOPS = 152 * 2 * 2.07 * 2
 # (the counters no longer describe the kernel that ran).
 #   M^-1 kernels: (config, precision, kernel) -> DRAM bytes of a launch
 #   Krylov kernels (work grows with the step j): -> (DRAM bytes, algorithmic bytes) of the captured step
-TRAFFIC_SOURCES = ["kernels.cu", "kernels.cuh", "ptx.cuh", "device.cu"]
+TRAFFIC_SOURCES = ["trsv.cu", "kernels.cu", "kernels.cuh", "stream.cuh", "lowrank.cuh", "ptx.cuh", "device.cu"]
 NCU_TRAFFIC_DIGEST = "916bf152ac449417"
 NCU_TRAFFIC = {
     ("c2", "mixed", "trsv_down_L0"): 43_714_560,
@@ -550,8 +550,8 @@ def run_ours(args):
 def level0_sweep_bytes(st, rows_total):
     """Bytes one level-0 sweep of the batched M^-1 must move (8 right-hand
     sides), from the batch's stats.  Each sweep is a solve with L and then U:
-    down: the chunks, the FP64 right-hand side in (64 B/row), the FP32 z1 out
-    (32 B/row); up: the chunks, F (values and columns 8 B per entry, row
+    down: the stored slices, the FP64 right-hand side in (64 B/row), the FP32 z1 out
+    (32 B/row); up: the slices, F (values and columns 8 B per entry, row
     offsets 8 B per row), the tail rows F reads (32 B/row), z1 in (32 B/row)
     and the FP64 result out (64 B/row)."""
     rows0 = st["lev0_rows"]

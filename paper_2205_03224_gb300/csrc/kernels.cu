@@ -1,7 +1,7 @@
 // CUDA kernels of the GeMSLR solve phase for sm_103a.
 //
 // Preconditioner application (Alg. 2), per Schur level l:
-//   k_trsv   (down)  z1 = U^-1 L^-1 b1          one CTA per diagonal block of B_l,
+//   k_trsv   (down)  z1 = U^-1 L^-1 b1          (trsv.cu) one CTA per diagonal block of B_l,
 //                    level-scheduled substitutions on a shared-memory copy of
 //                    the block's vector (Sec. 4.2: the p block solves are
 //                    independent);
