@@ -151,7 +151,7 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
 // The substitutions of one block for RPC right-hand sides, the vector in shared
 // memory.  Bound by the chain of wavefronts (a 48^3 system's first-level block:
 // about 640 of 20 to 60 rows), so, as in the single-system kernels, a set of warps
-// has its next rows in registers when their wavefront is due, two sets take the
+// has its next rows in registers when their wavefront is due, four sets take the
 // slices in turn, a barrier ends every wavefront, and nothing on the chain
 // branches.  A lane holds four right-hand sides of one row: an entry costs it
 // one 16-byte gather and four FMAs.  MODE as in k_btrsv; the rows' sums too (even

@@ -33,7 +33,11 @@ namespace gemslr {
 namespace {
 
 // z2 = b2 - E z1 on rows [row0, row1) of the tail, then partial W^T z2 (W^H z2
-// for the complex hierarchy).
+// for the complex hierarchy).  Bound by the chain of memory round trips (row
+// extents, entries, x, the partials' hand-over) and by FP64 additions, which hold
+// an SM quarter for 64 cycles each: so W is requested first and no zero is added.
+// 32 x 32, FP64 (one CTA of 63 rows): 14 -> 10.5 us; 64^3 mixed 11 to 13 us a level,
+// FP64 18 to 19, where the hand-over between CTAs dominates.
 template <typename VT, typename WT>
 __global__ void __launch_bounds__(kCoupleRows)
 k_couple(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restrict__ work,
