@@ -486,10 +486,12 @@ uint64_t gemslr_kernel_launches(void);
  * gemslr_selftest_wait (no counterpart in the paper): exercises the bounded
  * device waits every staged kernel relies on.  One CTA waits on an mbarrier
  * that nothing completes, once with the suspending wait and once with the
- * polling wait, each bounded by `cycles` SM clock cycles (> 0).  Returns
- * GEMSLR_ERR_TIMEOUT when both waits gave up and the context is still usable
+ * polling wait, each bounded by `cycles` SM clock cycles (> 0); a third warp
+ * polls an mbarrier that completes after the bound of half of its lanes.  Returns
+ * GEMSLR_ERR_TIMEOUT when both waits gave up, the third warp's lanes were all
+ * told the same and the context is still usable
  * afterwards (the expected outcome), GEMSLR_ERR_CUDA on a CUDA error,
- * GEMSLR_ERR_ARG if a wait returned or cycles <= 0.  Uses the default stream
+ * GEMSLR_ERR_ARG if a wait returned, the lanes disagree or cycles <= 0.  Uses the default stream
  * and synchronises the device.
  */
 gemslr_status gemslr_selftest_wait(int64_t cycles);

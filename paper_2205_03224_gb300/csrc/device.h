@@ -92,7 +92,7 @@ void prepare_krylov_kernels();
 void launch_dgs_close(int64_t len, const double *V, int64_t ldv, const double *vt, double *partial, unsigned *counter,
                       KrylovCtl *ctl, const DgsBufs &B, int grid, cudaStream_t st);
 void launch_lsq2(const KrylovCtl *ctl, const double *H, const double *g, const double *R, double *y, cudaStream_t st);
-// Two bounded waits on an mbarrier nothing completes (see gemslr_selftest_wait).
+// Bounded waits that expire: two whole warps, and half of the lanes of a third (see gemslr_selftest_wait).
 void launch_wait_selftest(long long limit, int32_t *gave_up, cudaStream_t st);
 void launch_norm2(int64_t len, const double *x, double *partial, unsigned *counter, double *out, int grid,
                   cudaStream_t st);

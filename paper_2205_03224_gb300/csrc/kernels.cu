@@ -151,19 +151,31 @@ k_couple(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restr
 // An mbarrier that nothing ever completes: warp 0 waits on it with the
 // suspending wait, warp 1 with the polling wait, both bounded by `limit`
 // clock cycles.  gave_up[w] = 1 when warp w's wait expired (it must).
+// Warp 2 polls a barrier that warp 0 completes when its own wait is over, half of
+// its lanes with a bound that ends before and half with one that ends after:
+// gave_up[2] = lanes that were told of an expired wait (all of them, or the warp
+// would part in what follows).
 __global__ void k_wait_selftest(long long limit, int32_t *gave_up) {
-    __shared__ uint64_t bar;
+    __shared__ uint64_t bar, late;
     __shared__ int abort_flag;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
+        mbar_init(&late, 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 2) {
+        const bool got = poll_warp(&late, 0, &abort_flag, lane < 16 ? limit / 2 : 4 * limit);
+        const int told = __popc(__ballot_sync(0xffffffffu, !got));
+        if (lane == 0) gave_up[warp] = told;
+        return;
+    }
     const bool got = warp == 0 ? wait_bounded(&bar, 0, &abort_flag, limit)
-                               : poll_bounded(&bar, 0, &abort_flag, limit);
-    if ((threadIdx.x & 31) == 0) gave_up[warp] = got ? 0 : 1;
+                               : poll_warp(&bar, 0, &abort_flag, limit);
+    if (lane == 0) gave_up[warp] = got ? 0 : 1;
+    if (threadIdx.x == 0) mbar_arrive(&late);
 }
 
 // ---- vectors ----------------------------------------------------------------
@@ -1350,7 +1362,7 @@ void launch_gs_scale(int64_t len, double *V, int64_t ldv, const double *w, const
     count_launch();
 }
 void launch_wait_selftest(long long limit, int32_t *gave_up, cudaStream_t st) {
-    k_wait_selftest<<<1, 64, 0, st>>>(limit, gave_up);
+    k_wait_selftest<<<1, 96, 0, st>>>(limit, gave_up);
     count_launch();
 }
 void launch_dgs_dots(int64_t len, const int64_t *rp, const int32_t *ci, const double *av, const double *z, double *zcol,

@@ -139,6 +139,14 @@ __device__ __forceinline__ bool poll_bounded(uint64_t *bar, unsigned parity, vol
     }
     return true;
 }
+// The same for a whole warp, with one outcome for all of its lanes: each lane has
+// its own clock and reads the abort flag at its own time, and lanes that went
+// different ways would wait for each other in the next shuffle, __syncwarp or
+// barrier for ever.
+__device__ __forceinline__ bool poll_warp(uint64_t *bar, unsigned parity, volatile int *abort_flag,
+                                          long long limit = kSpinCycles) {
+    return __all_sync(0xffffffffu, poll_bounded(bar, parity, abort_flag, limit));
+}
 // One bulk copy global -> shared (16-byte aligned addresses, size a multiple of
 // 16).  The factor chunks are read once per application, so the copy marks
 // them evict-first in L2: the vectors that the substitutions gather from (in
@@ -219,11 +227,12 @@ __device__ __forceinline__ void produce_chunks(const unsigned char *data, const 
             wait_bounded(&full[g % kMaxSlots], (g / kMaxSlots) & 1, nullptr);
 }
 
-// Wait until chunk k (block-relative) is in shared memory and return it (nullptr: the wait expired).
+// Wait until chunk k (block-relative) is in shared memory and return it (nullptr, in
+// every lane: the wait expired).
 __device__ __forceinline__ const unsigned char *wait_chunk(const unsigned char *ring, uint64_t *full,
                                                            volatile int *abort_flag, int k) {
     const int slot = k % kMaxSlots;
-    return poll_bounded(&full[slot], (k / kMaxSlots) & 1, abort_flag) ? ring + (size_t)slot * kStageBytes : nullptr;
+    return poll_warp(&full[slot], (k / kMaxSlots) & 1, abort_flag) ? ring + (size_t)slot * kStageBytes : nullptr;
 }
 
 }  // namespace

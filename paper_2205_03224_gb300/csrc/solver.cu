@@ -1290,21 +1290,22 @@ gemslr_status gemslr_selftest_wait(int64_t cycles) {
     return guard([&] {
         if (cycles <= 0) fail(GEMSLR_ERR_ARG, "cycles must be positive");
         int32_t *dev = nullptr;
-        GEMSLR_CUDA(cudaMalloc(&dev, 2 * sizeof(int32_t)));
-        int32_t host[2] = {0, 0};
-        cudaError_t e = cudaMemset(dev, 0, 2 * sizeof(int32_t));
+        GEMSLR_CUDA(cudaMalloc(&dev, 3 * sizeof(int32_t)));
+        int32_t host[3] = {0, 0, 0};
+        cudaError_t e = cudaMemset(dev, 0, 3 * sizeof(int32_t));
         if (e == cudaSuccess) {
             launch_wait_selftest((long long)cycles, dev, 0);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaMemcpy(host, dev, sizeof(host), cudaMemcpyDeviceToHost);
         // the context must still be usable after the expired waits
-        if (e == cudaSuccess) e = cudaMemset(dev, 0, 2 * sizeof(int32_t));
+        if (e == cudaSuccess) e = cudaMemset(dev, 0, 3 * sizeof(int32_t));
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         cudaFree(dev);
         if (e != cudaSuccess) fail(GEMSLR_ERR_CUDA, cudaGetErrorString(e));
         if (host[0] != 1 || host[1] != 1) fail(GEMSLR_ERR_ARG, "a wait on an mbarrier that nothing completes returned");
-        fail(GEMSLR_ERR_TIMEOUT, "bounded waits expired as expected (self-test)");
+        if (host[2] != 32) fail(GEMSLR_ERR_ARG, "the lanes of a warp disagree on whether a wait expired");
+        fail(GEMSLR_ERR_TIMEOUT, "bounded waits expired as expected, for all lanes of a warp alike (self-test)");
     });
 }
 

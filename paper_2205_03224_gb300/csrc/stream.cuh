@@ -147,9 +147,9 @@ struct ItemWalk {
 
     __device__ ItemWalk(const StreamView &S, StreamHead *h, const unsigned char *r, int consumer)
         : H(h), ring(smem_u32(r)), slots(S.slots), slot_bytes(S.slot_bytes), step(S.consumers), slot(consumer) {}
-    // Shared address of the current item, once it has arrived (0: the bounded wait expired).
+    // Shared address of the current item, once it has arrived (0, in every lane: the bounded wait expired).
     __device__ __forceinline__ uint32_t item() {
-        if (!poll_bounded(&H->full[slot], parity, &H->abort_flag)) {
+        if (!poll_warp(&H->full[slot], parity, &H->abort_flag)) {
             *(volatile int *)&H->abort_flag = 1;
             return 0;
         }

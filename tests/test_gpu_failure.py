@@ -35,3 +35,12 @@ def test_bounded_waits_expire_and_context_survives(torch_cuda):
 def test_selftest_rejects_bad_argument(torch_cuda):
     from paper_2205_03224_gb300 import _lib
     assert _lib.selftest_wait(0) == "ERR_ARG"
+
+
+@pytest.mark.parametrize("cycles", [100_000, 2_000_000])
+def test_expired_wait_is_one_outcome_for_all_lanes(torch_cuda, cycles):
+    """A wait that runs out for half of a warp's lanes only: the kernels' next
+    full-warp operation needs all of them on the same path."""
+    from paper_2205_03224_gb300 import _lib
+    assert _lib.selftest_wait(cycles) == "ERR_TIMEOUT"
+    assert "all lanes of a warp alike" in _lib.load().gemslr_last_error().decode()
