@@ -161,7 +161,9 @@ __device__ __forceinline__ void consume_long_rows(ItemWalk &W, const X &x, int l
             const int2 e = lds<int2>(p);
             if (e.x >= 0) a0 += __int_as_float(e.y) * x.load(e.x);
         }
-        x.store(R.row, fmaf(self, R.dinv, sum_rn(a0, a1)));
+        // lanes past the last row hold it too: they must not store, another of them
+        // may still have its x_i to read
+        if (lane <= h.x) x.store(R.row, fmaf(self, R.dinv, sum_rn(a0, a1)));
         W.next(lane);
     }
 }
