@@ -38,6 +38,16 @@ __device__ __forceinline__ bool last_of(unsigned *counter, unsigned n) {
 // right-hand side from `in` (FP64) or `work`.  MODE 1: right-hand side F y2,
 // then work[rows] -= result.  Without SMEM (blocks too large even for RPC = 1)
 // RPC is kBatchRhs and the vector stays in global memory.
+// Bound by a row's gathers, one chunk of rows after another: four entries (shared
+// memory) or six (global memory) are in flight at a time, written out because the
+// compiler's own choice changes with the code around it, and the next chunk is
+// looked for before the sums.  In global memory the gathers have to hit in L1, so
+// the carve-out leaves it all but two CTAs' rings (set_btrsv_smem_limit): when the
+// kernel takes only 32 registers a third CTA would fit, the driver gives shared
+// memory the whole SM for it, and an application of 8 systems of 56^3 took 4.18 ms
+// instead of 2.68.  Now 2.58; 96 systems (sides 16 to 48), rows of up to 20 entries,
+// 5.50 ms (7.68; with 48 registers and no such figure 5.55); 24 of them (10 to 20), in
+// shared memory, 0.71 (0.72).
 template <int MODE, bool SMEM, int RPC>
 __global__ void __launch_bounds__(kBatchTrsvThreads)
 k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ work, double *__restrict__ out_final,
@@ -90,16 +100,17 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
         }
     }
     batch_consumer_barrier();
-    bool aborted = false;
+    bool aborted = false, ready = false;
     const int rr = lane / RPC, r = lane % RPC;
     for (int c = c0; c < c1; ++c) {
         const int k = c - c0;
-        const unsigned char *base = aborted ? nullptr : wait_chunk(ring, full, abort_flag, k);
+        const unsigned char *base = aborted ? nullptr : wait_chunk(ring, full, abort_flag, k, ready);
         if (!aborted && !base) {
             aborted = true;
             *abort_flag = 1;
         }
         if (!aborted) {
+            const bool next = c + 1 < c1 && chunk_ready(full, k + 1);
             const int *hdr = reinterpret_cast<const int *>(base);
             const int nrow = hdr[0], S = hdr[1], upper = hdr[2];
             const int pr = (nrow + 3) & ~3;
@@ -118,15 +129,43 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
                 const float self = xs[row * RPC + r], d = upper ? dinv[t] : 1.f;
                 float a0 = 0.f, a1 = 0.f;
                 int q = 0;
-                for (; q + 1 < len; q += 2) {
-                    a0 += vals[q * nrow + t] * xs[cols[q * nrow + t] * RPC + r];
-                    a1 += vals[(q + 1) * nrow + t] * xs[cols[(q + 1) * nrow + t] * RPC + r];
+                if constexpr (SMEM) {
+#pragma unroll 1
+                    for (; q + 3 < len; q += 4) {
+                        float v[4], x[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            v[u] = vals[(q + u) * nrow + t];
+                            x[u] = xs[cols[(q + u) * nrow + t] * RPC + r];
+                        }
+                        a0 += v[0] * x[0];
+                        a1 += v[1] * x[1];
+                        a0 += v[2] * x[2];
+                        a1 += v[3] * x[3];
+                    }
+                    float v[3], x[3];                        // the last one to three, absent ones 0 * 0
+#pragma unroll
+                    for (int u = 0; u < 3; ++u) {
+                        const bool on = q + u < len;
+                        v[u] = on ? vals[(q + u) * nrow + t] : 0.f;
+                        x[u] = on ? xs[cols[(q + u) * nrow + t] * RPC + r] : 0.f;
+                    }
+                    a0 += v[0] * x[0];
+                    a1 += v[1] * x[1];
+                    a0 += v[2] * x[2];
+                } else {
+#pragma unroll 3
+                    for (; q + 1 < len; q += 2) {
+                        a0 += vals[q * nrow + t] * xs[cols[q * nrow + t] * RPC + r];
+                        a1 += vals[(q + 1) * nrow + t] * xs[cols[(q + 1) * nrow + t] * RPC + r];
+                    }
+                    if (q < len) a0 += vals[q * nrow + t] * xs[cols[q * nrow + t] * RPC + r];
                 }
-                if (q < len) a0 += vals[q * nrow + t] * xs[cols[q * nrow + t] * RPC + r];
                 xs[row * RPC + r] = fmaf(self, d, a0 + a1);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[k % kSlots]);
+            ready = __all_sync(0xffffffffu, next);
         }
         batch_consumer_barrier();
     }
@@ -1072,6 +1111,11 @@ void set_btrsv_smem_limit(int bytes) {
     set_btrsv_attr<1>(bytes);
     cudaFuncSetAttribute(k_btrsv<0, false, R8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
     cudaFuncSetAttribute(k_btrsv<1, false, R8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    // vectors in global memory: two CTAs' rings in 132 of the SM's 228 KB, the rest is L1 (a rounded-up
+    // percentage would take 164)
+    for (auto kernel : {k_btrsv<0, false, R8>, k_btrsv<1, false, R8>})
+        cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             100 * 2 * (kRingBytes + 1024) / (228 * 1024));
 }
 void launch_bcouple(const BatchLevel &lv, const double *in, float *work, cudaStream_t st) {
     if (lv.ncta == 0) return;

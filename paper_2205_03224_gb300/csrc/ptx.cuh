@@ -227,12 +227,16 @@ __device__ __forceinline__ void produce_chunks(const unsigned char *data, const 
             wait_bounded(&full[g % kMaxSlots], (g / kMaxSlots) & 1, nullptr);
 }
 
-// Wait until chunk k (block-relative) is in shared memory and return it (nullptr, in
-// every lane: the wait expired).
+// Whether chunk k (block-relative) is in shared memory, by this lane's look.
+__device__ __forceinline__ bool chunk_ready(uint64_t *full, int k) {
+    return mbar_test_wait(&full[k % kMaxSlots], (k / kMaxSlots) & 1);
+}
+// Wait until chunk k is in shared memory, unless it is known to be (ready: every lane
+// has seen it), and return it (nullptr, in every lane: the wait expired).
 __device__ __forceinline__ const unsigned char *wait_chunk(const unsigned char *ring, uint64_t *full,
-                                                           volatile int *abort_flag, int k) {
+                                                           volatile int *abort_flag, int k, bool ready) {
     const int slot = k % kMaxSlots;
-    return poll_warp(&full[slot], (k / kMaxSlots) & 1, abort_flag) ? ring + (size_t)slot * kStageBytes : nullptr;
+    return ready || poll_warp(&full[slot], (k / kMaxSlots) & 1, abort_flag) ? ring + (size_t)slot * kStageBytes : nullptr;
 }
 
 }  // namespace

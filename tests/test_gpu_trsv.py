@@ -150,3 +150,26 @@ def test_partial_slices_give_the_same_bits_every_time(name):
         assert torch.equal(G.apply(rd), z)
     ref = _solved(blocks, sizes, r)
     assert np.max(np.abs(z.cpu().numpy() - ref)) <= 3e-5 * np.max(np.abs(ref))
+
+
+# Batched levels that are not streamed (a block beyond shared memory even for four
+# right-hand sides, with and without rows longer than a record): the right-hand sides
+# split over CTAs while these run in one wave, else vectors in global memory.
+CASES.update(large_block=([13000, 4000], 7, 900, False), large_block_long_rows=([13000, 4000], 20, 60, False))
+
+
+@pytest.mark.parametrize("nsys,per_cta", [(3, 2), (24, 0)])
+@pytest.mark.parametrize("name", ["large_block", "large_block_long_rows"])
+def test_batched_large_blocks_against_plain_solves(name, nsys, per_cta):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_03224_gb300 import GemslrBatch
+    rng, blocks, sizes, A, part, fac = _system(name, False)
+    B = GemslrBatch.from_factors([A] * nsys, [part] * nsys, [fac] * nsys)
+    assert B.stats()["rhs_per_cta"] == per_cta
+    r = rng.uniform(-1, 1, (nsys, 8, A.n))
+    z = B.apply(torch.from_numpy(r.ravel()).cuda(), 8).cpu().numpy().reshape(r.shape)
+    for s, q in ((0, 0), (0, 7), (1, 3), (nsys - 1, 0), (nsys - 1, 7)):
+        ref = _solved(blocks, sizes, r[s, q])
+        assert np.max(np.abs(z[s, q] - ref)) <= 3e-5 * np.max(np.abs(ref)), (s, q)
