@@ -314,16 +314,16 @@ std::vector<SliceRows> cut_slices(const Waves &W, int64_t r0, bool upper, int64_
 
 struct EntryF32 { int32_t col; float v; };
 
-// FP32 row i into its record of np pairs: pair p at slot(p), entries from 16 on to rest[(e - 16) * step].
+// FP32 row i into its record of np pairs: pair p at slot(p), entries from 16 on to rest.
 template <typename Slot>
-void put_row_f32(const Csr &T, int64_t r0, int64_t i, bool upper, EntryF32 *rec, Slot slot, EntryF32 *rest, int64_t step) {
+void put_row_f32(const Csr &T, int64_t r0, int64_t i, bool upper, EntryF32 *rec, Slot slot, EntryF32 *rest) {
     const int64_t pdiag = upper ? diagonal(T, i) : -1;
     int64_t e = 0;
     for (int64_t p = T.rp[i]; p < T.rp[i + 1]; ++p) {
         if (T.ci[p] == i) continue;
         const EntryF32 en{(int32_t)((T.ci[p] - r0) * 4), stored_entry<float>(T, p, pdiag)};
         if (e < 16) rec[2 * slot(e / 2) + e % 2] = en;
-        else rest[(e - 16) * step] = en;
+        else rest[e - 16] = en;
         ++e;
     }
 }
@@ -331,35 +331,69 @@ EntryF32 row_head_f32(const Csr &T, int64_t r0, int64_t i, bool upper) {
     return {(int32_t)((i - r0) * 4), upper ? inv_entry<float>(T, diagonal(T, i)) : 1.f};
 }
 
-// FP32: rows to their heads and records; entries from 16 on to rest.
+// FP32: rows to their heads and records of np pairs, entries from 16 on to their rests.
 void put_rows_f32(const Csr &T, int64_t r0, const Waves &W, bool upper, const int64_t *rows, int64_t n, int np,
-                  unsigned char *p) {
+                  unsigned char *p, unsigned char *rest, size_t rest_bytes) {
     EntryF32 *head = reinterpret_cast<EntryF32 *>(p);
     unsigned char *recs = p + pad16((size_t)(8 * n));
-    const bool longer = np == kLongRows;
-    const int pairs = longer ? 8 : np;
-    EntryF32 *rest = reinterpret_cast<EntryF32 *>(recs + row_bytes(pairs) * n);
     for (int64_t t = 0; t < n; ++t) {
-        const int64_t i = rows[t], shift = longer ? 0 : pairs - (W.len[i - r0] + 1) / 2;
+        const int64_t i = rows[t], shift = np - (std::min<int64_t>(16, W.len[i - r0]) + 1) / 2;
         head[t] = row_head_f32(T, r0, i, upper);
-        put_row_f32(T, r0, i, upper, reinterpret_cast<EntryF32 *>(recs + row_bytes(pairs) * t),
-                    [&](int64_t pr) { return upper && !longer ? pairs - 1 - pr : pr + shift; }, rest + t, n);
+        put_row_f32(T, r0, i, upper, reinterpret_cast<EntryF32 *>(recs + row_bytes(np) * t),
+                    [&](int64_t pr) { return upper ? np - 1 - pr : pr + shift; },
+                    reinterpret_cast<EntryF32 *>(rest + rest_bytes * t));
     }
 }
 
-// FP32, rows of at most 16 entries: groups of four slices.
+// Slices of FP32 rows, cut further where their entries from 16 on would fill more than a
+// third of an item.
+struct SliceF32 {
+    const int64_t *rows;
+    int64_t n, quads = 0;              // rows; fours of entries from 16 on
+    size_t bytes(int np) const { return pad16((size_t)(8 * n)) + (size_t)(row_bytes(np) * n); }
+    size_t rests() const { return quads ? (size_t)(rest_bytes((int)quads) * n) : 0; }
+};
+std::vector<SliceF32> cut_f32(const Waves &W, int64_t r0, bool upper, int np, bool longer) {
+    std::vector<SliceF32> out;
+    for (const SliceRows &s : cut_slices<float>(W, r0, upper, np == 8 ? 24 : 32))      // four fit kMaxItemBytes
+        for (int64_t at = 0; at < s.n; at += out.back().n) {
+            SliceF32 c{s.rows + at, s.n - at};
+            if (longer) {
+                const int64_t longest = W.len[s.rows[at] - r0];
+                c.quads = std::max<int64_t>(0, longest - 16 + 3) / 4;
+                while (c.n > 1 && c.bytes(np) + c.rests() > (size_t)kMaxItemBytes / 3 - 64) --c.n;
+            }
+            out.push_back(c);
+        }
+    return out;
+}
+
+// FP32: groups of four slices of one factor (see kernels.cuh).
 void append_groups(const Csr &T, int64_t r0, const Waves &W, bool upper, StreamHost &out) {
-    const int np = out.np;
-    const std::vector<SliceRows> sl = cut_slices<float>(W, r0, upper, np == 8 ? 24 : 32);   // four fit kMaxItemBytes
-    // the sequence of slices; -1: without rows (see kernels.cuh)
+    const bool longer = out.np == kLongRows;
+    const int np = longer ? 8 : out.np, header = longer ? 2 * kItemHeader : kItemHeader;
+    const std::vector<SliceF32> sl = cut_f32(W, r0, upper, np, longer);
+    // the sequence of slices; -1: without rows
     std::vector<int64_t> seq;
     std::vector<int32_t> slice_of(W.len.size(), -1);
+    auto bytes = [&](int64_t k) { return k < 0 ? SliceF32{nullptr, 1}.bytes(np) : sl[k].bytes(np) + sl[k].rests(); };
+    size_t total = header;             // of the last group
+    auto push = [&](int64_t k) {
+        if (seq.size() % 4 == 0) total = header;
+        // a long row's slice that does not fit beside the others starts a group
+        while (total + bytes(k) + (3 - seq.size() % 4) * bytes(-1) > (size_t)kMaxItemBytes && seq.size() % 4) {
+            seq.push_back(-1);
+            total = seq.size() % 4 ? total + bytes(-1) : header;
+        }
+        seq.push_back(k);
+        total += bytes(k);
+    };
     for (size_t k = 0; k < sl.size(); ++k) {
         int64_t late = 0;
         for (int64_t t = 0; k > 0 && t < sl[k].n; ++t) {
-            const int64_t i = sl[k].rows[t], len = W.len[i - r0];
+            const int64_t i = sl[k].rows[t], len = std::min<int64_t>(16, W.len[i - r0]);
             int64_t e = 0;
-            for (int64_t p = T.rp[i]; p < T.rp[i + 1]; ++p) {
+            for (int64_t p = T.rp[i]; p < T.rp[i + 1] && e < 16; ++p) {
                 if (T.ci[p] == i) continue;
                 if (slice_of[T.ci[p] - r0] == (int32_t)k - 1)
                     late = std::max(late, upper ? e / 2 + 1 : (len + 1) / 2 - e / 2);
@@ -367,46 +401,29 @@ void append_groups(const Csr &T, int64_t r0, const Waves &W, bool upper, StreamH
             }
         }
         for (int64_t t = 0; t < sl[k].n; ++t) slice_of[sl[k].rows[t] - r0] = (int32_t)k;
-        if (late > kLatePairs || (upper && k == 0)) seq.push_back(-1);
-        seq.push_back((int64_t)k);
+        if (late > kLatePairs || (upper && k == 0)) push(-1);
+        push((int64_t)k);
     }
     while (seq.size() % 4) seq.push_back(-1);
-    auto rows = [&](int64_t k) { return k < 0 ? 1 : sl[k].n; };
     for (size_t g = 0; g < seq.size(); g += 4) {
-        size_t total = kItemHeader;
-        for (size_t q = g; q < g + 4; ++q) total += pad16((size_t)(8 * rows(seq[q]))) + (size_t)(row_bytes(np) * rows(seq[q]));
-        const size_t item = add_item(out, total);
+        size_t all = header;
+        for (size_t q = g; q < g + 4; ++q) all += bytes(seq[q]);
+        const size_t item = add_item(out, all);
         unsigned char *p = out.data.data() + item;
-        size_t off = kItemHeader;
+        int32_t *h = reinterpret_cast<int32_t *>(p);
+        size_t off = header;
         for (size_t q = g; q < g + 4; ++q) {
-            const int64_t k = seq[q], n = rows(k);
-            reinterpret_cast<int32_t *>(p)[q - g] = (int32_t)(off << 16) | (int32_t)(n - 1);
+            const int64_t k = seq[q];
+            const SliceF32 c = k < 0 ? SliceF32{nullptr, 1} : sl[k];
+            h[q - g] = (int32_t)(off << 16) | (int32_t)(c.n - 1);
+            unsigned char *rest = p + off + c.bytes(np);
+            if (c.quads) {
+                h[4 + q - g] = (int32_t)(off + c.bytes(np)) | (int32_t)(c.quads << kRestQuads);
+                for (size_t e = 0; e < c.rests() / sizeof(EntryF32); ++e) reinterpret_cast<EntryF32 *>(rest)[e] = {kNoEntry, 0.f};
+            }
             if (k < 0) *reinterpret_cast<EntryF32 *>(p + off) = {kNoRow, 1.f};
-            else put_rows_f32(T, r0, W, upper, sl[k].rows, n, np, p + off);
-            off += pad16((size_t)(8 * n)) + (size_t)(row_bytes(np) * n);
-        }
-    }
-}
-
-// FP32, any rows: one slice per item.
-void append_long_rows(const Csr &T, int64_t r0, const Waves &W, bool upper, StreamHost &out) {
-    auto bytes = [&](int64_t n, int64_t z) {
-        return kItemHeader + pad16((size_t)(8 * n)) + (size_t)((row_bytes(8) + 8 * z) * n);
-    };
-    for (const SliceRows &s : cut_slices<float>(W, r0, upper, 32)) {
-        const int64_t z = std::max<int64_t>(0, s.longest - 16);
-        for (int64_t at = 0; at < s.n;) {
-            int64_t n = 1;
-            while (at + n < s.n && bytes(n + 1, z) <= (size_t)kMaxItemBytes) ++n;
-            const size_t item = add_item(out, bytes(n, z));
-            int32_t *h = reinterpret_cast<int32_t *>(out.data.data() + item);
-            h[0] = (int32_t)n - 1;
-            h[2] = (int32_t)z;
-            unsigned char *p = out.data.data() + item + kItemHeader;
-            EntryF32 *rest = reinterpret_cast<EntryF32 *>(p + pad16((size_t)(8 * n)) + row_bytes(8) * n);
-            for (int64_t k = 0; k < z * n; ++k) rest[k] = {-1, 0.f};
-            put_rows_f32(T, r0, W, upper, s.rows + at, n, kLongRows, p);
-            at += n;
+            else put_rows_f32(T, r0, W, upper, c.rows, c.n, np, p + off, rest, rest_bytes((int)c.quads));
+            off += bytes(k);
         }
     }
 }
@@ -581,15 +598,14 @@ void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, St
     out.np = trsv_record(one, longest);
     int64_t nwave = 1;
     for (size_t b = 0; b < nb; ++b) nwave += (int64_t)(wl[b].ptr.size() + wu[b].ptr.size());
-    out.consumers = !one ? trsv_sets((double)(2 * bp.back()) / (double)(nwave * kLaneRows<VT>)) : out.np == kLongRows ? 1 : 4;
+    out.consumers = !one ? trsv_sets((double)(2 * bp.back()) / (double)(nwave * kLaneRows<VT>)) : 4;
     for (size_t b = 0; b < nb; ++b) {
         const int64_t r0 = bp[b];
         if constexpr (one) {
             const size_t first = out.off.size();
-            auto append = out.np == kLongRows ? append_long_rows : append_groups;
-            append(L, r0, wl[b], false, out);
+            append_groups(L, r0, wl[b], false, out);
             out.split.push_back((int32_t)(out.off.size() - first));
-            append(U, r0, wu[b], true, out);
+            append_groups(U, r0, wu[b], true, out);
         } else {
             LaneSlices s;
             append_lanes<VT>(L, r0, wl[b], false, out.np, s);

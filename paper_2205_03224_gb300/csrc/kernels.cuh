@@ -28,15 +28,17 @@ constexpr int kMaxCols = 160;     // Krylov columns per Gram-Schmidt pass (m + 1
 // those from 16 on, a1 that of the odd ones below 16, in order; one lane per row,
 // slices of at most 32 rows.  {row, d}[rows], padded to 16 bytes, then
 // row_bytes(np) per row: np pairs of entries (column, value), absent ones (0, 0).
-// Levels whose rows have at most 16 entries: an item is a group of four slices of
+// An item is a group of four slices of
 // one factor, four int32 {rows - 1, offset in the high half}, then the slices; four
 // consumer warps.  L's records end with the row's last pair; U's hold the pairs in
 // reverse.  So the entries of the slice just before, the nearest columns, sit in
 // the last kLatePairs pairs: a slice of one row at kNoRow separates slices that
 // need more, and L from U, and fills a factor's last group.
-// Levels with longer rows (np = kLongRows): one slice per item, one consumer
-// warp; header int32 {rows - 1, 0, z, 0}, the slice with np = 8, and {column,
-// value}[z][rows] for the entries from 16 on (absent: column -1).
+// Levels with rows of more than 16 entries (np = kLongRows): records of 8 pairs for the
+// first 16, four more int32 in the item's header {offset of the slice's rests, fours
+// of entries in the longest << kRestQuads} (0: none) and, behind each slice's records,
+// rest_bytes(quads) per row for its entries from 16 on, absent ones (kNoEntry, 0).
+// They may come from the slice just before.
 //
 // FP64 and complex: four chains per row, a row's entry e in chain e % 4 (a lane;
 // two in complex arithmetic); chain
@@ -63,9 +65,10 @@ template <typename VT> constexpr int kLaneRows = sizeof(VT) == 8 ? 32 : 16;   //
 constexpr int kMaxItemBytes = 16192;            // head and a slot for each of four consumers within kRingBytes
 constexpr int kItemDepth = 16;                  // most slots per consumer
 constexpr int kLatePairs = 3;
-constexpr int kNoRow = -4;
+constexpr int kNoRow = -4, kNoEntry = -8;      // places in the StreamHead
 constexpr int kLaneItemBytes = 8192;            // FP64: slices of a consumer are joined into items of about this size
 constexpr int kLongRows = 16;
+constexpr int kRestQuads = 16;
 enum { kSync = 1 };
 // class of a slice (flags >> kLaneShift & 7): longest row 1, 2, up to 4 entries, more, more than 16; scaling
 enum { kLaneShift = 4, kLane1 = 0, kLane2, kLane4, kLaneFull, kLaneLong, kLaneScale };
@@ -73,6 +76,7 @@ template <typename VT> struct OneLaneRows { static constexpr bool value = false;
 template <> struct OneLaneRows<float> { static constexpr bool value = true; };
 __host__ __device__ constexpr int odd16(int bytes) { return (((bytes + 15) / 16) | 1) * 16; }
 __host__ __device__ constexpr int row_bytes(int np) { return odd16(16 * np); }
+__host__ __device__ constexpr int rest_bytes(int quads) { return odd16(32 * quads); }
 template <typename VT>
 __host__ __device__ constexpr int lane_bytes(int kq) { return odd16(kq * ((int)sizeof(VT) + 4) + 4); }
 
@@ -80,7 +84,8 @@ __host__ __device__ constexpr int lane_bytes(int kq) { return odd16(kq * ((int)s
 // that ends every wait of the CTA; the block's vector and the ring follow.
 struct StreamHead {
     uint64_t full[4 * kItemDepth], empty[4 * kItemDepth];
-    int abort_flag, pad[3];
+    int abort_flag, pad;
+    float no_entry, no_row;    // FP32: zero, for absent entries; the slot of slices without rows
 };
 static_assert(sizeof(StreamHead) % 16 == 0 && (int)sizeof(StreamHead) + 4 * kMaxItemBytes <= kRingBytes, "smallest ring");
 
@@ -90,7 +95,7 @@ struct StreamView {
     const int32_t *blk_item;   // nblk + 1 item range of every block
     const int32_t *split;      // nblk: items of L (FP32), slices with kSync (FP64)
     int32_t np;                // pairs per row record (FP32), entries per lane record (FP64)
-    int32_t consumers;         // FP32: 4, 1 for long rows; FP64: 2 or 4
+    int32_t consumers;         // FP32: 4; FP64: 2 or 4
     int32_t slots, slot_bytes; // the ring
 };
 

@@ -97,8 +97,7 @@ template <> __device__ __forceinline__ int4 lds<int4>(uint32_t a) {
 }
 // The block's vector by byte offset, in shared memory (right behind the
 // StreamHead: a constant address, so that a gather needs no addition) or in
-// global memory.  Offset kNoRow (the StreamHead's last word): the slot of slices
-// without rows.
+// global memory.  Offsets kNoRow and kNoEntry: words of the StreamHead.
 template <typename VT, bool SMEM>
 struct BlockVec;
 template <typename VT>
@@ -111,6 +110,7 @@ struct BlockVec<VT, true> {
     __device__ __forceinline__ VT load(int off) const {
         return *reinterpret_cast<const VT *>(reinterpret_cast<const unsigned char *>(vec()) + off);
     }
+    __device__ __forceinline__ VT load_entry(int off) const { return load(off); }
     __device__ __forceinline__ void store(int off, VT v) const {
         *reinterpret_cast<VT *>(reinterpret_cast<unsigned char *>(vec()) + off) = v;
     }
@@ -127,6 +127,10 @@ struct BlockVec<VT, false> {
     unsigned char *base;
     __device__ explicit BlockVec(VT *x) : base(reinterpret_cast<unsigned char *>(x)) {}
     __device__ __forceinline__ VT load(int off) const { return *reinterpret_cast<const VT *>(base + max(off, 0)); }
+    // x at an entry's column, 0 at kNoEntry
+    __device__ __forceinline__ VT load_entry(int off) const {
+        return off >= 0 ? *reinterpret_cast<const VT *>(base + off) : (VT)0;
+    }
     __device__ __forceinline__ void store(int off, VT v) const {
         if (off >= 0) *reinterpret_cast<VT *>(base + off) = v;
     }

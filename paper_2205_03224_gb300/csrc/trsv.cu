@@ -65,9 +65,10 @@ __device__ __forceinline__ void gather_f32(const RowF32<NP> &R, const X &x, floa
     }
 }
 
-// The row's sum over its pairs in order (DOWN: the record holds them in reverse).
-template <int NP, bool DOWN>
-__device__ __forceinline__ float row_f32(const RowF32<NP> &R, const float *xv, float self) {
+// The row's sum over its pairs in order (DOWN: the record holds them in reverse);
+// rest: what follows them in the sum of the even ones.
+template <int NP, bool DOWN, typename Rest>
+__device__ __forceinline__ float row_f32(const RowF32<NP> &R, const float *xv, float self, Rest rest) {
     float a0 = 0, a1 = 0;
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
@@ -75,8 +76,48 @@ __device__ __forceinline__ float row_f32(const RowF32<NP> &R, const float *xv, f
         a0 += __int_as_float(R.e[i].y) * xv[2 * i];
         a1 += __int_as_float(R.e[i].w) * xv[2 * i + 1];
     }
-    return fmaf(self, R.dinv, sum_rn(a0, a1));
+    return fmaf(self, R.dinv, sum_rn(rest(a0), a1));
 }
+
+// A row's entries from 16 on (desc: see kernels.cuh), read from the staged item four
+// at a time: while four are added the next four x are gathered and the four entries
+// after them read; e: the first four, read ahead.  Bound by instructions, so absent
+// entries are added like the others.
+struct RestF32 {
+    int4 e[2];
+    uint32_t q;
+    __device__ __forceinline__ void fetch(uint32_t item, int desc, int t) {
+        q = item + (desc & ((1 << kRestQuads) - 1)) + rest_bytes(desc >> kRestQuads) * t;
+        e[0] = lds<int4>(q);
+        e[1] = lds<int4>(q + 16);
+    }
+    template <typename X>
+    __device__ __forceinline__ float add(int desc, const X &x, float a) {
+        int left = desc >> kRestQuads;
+        if (left == 0) return a;
+        const uint32_t end = q + 32 * (left - 1);
+        float v[4], xv[4];
+        auto gather = [&] {                         // x of the four in e, then the four after them
+            v[0] = __int_as_float(e[0].y), v[1] = __int_as_float(e[0].w);
+            v[2] = __int_as_float(e[1].y), v[3] = __int_as_float(e[1].w);
+            xv[0] = x.load_entry(e[0].x), xv[1] = x.load_entry(e[0].z);
+            xv[2] = x.load_entry(e[1].x), xv[3] = x.load_entry(e[1].z);
+            q = min(q + 32, end);
+            e[0] = lds<int4>(q);
+            e[1] = lds<int4>(q + 16);
+        };
+        gather();
+        for (; left > 1; --left) {
+            const float v0[4] = {v[0], v[1], v[2], v[3]}, x0[4] = {xv[0], xv[1], xv[2], xv[3]};
+            gather();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a = __fmaf_rn(v0[u], x0[u], a);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a = __fmaf_rn(v[u], xv[u], a);
+        return a;
+    }
+};
 
 // Named barriers that pass the sweep from the warp of one group to the warp of
 // the next (64 threads: one warp arrives, the other waits): kEarly + w tells
@@ -96,7 +137,13 @@ __device__ __forceinline__ void give_turn(int id) { asm volatile("bar.arrive %0,
 // as a gather): every group has four slices.  Every warp goes through the same
 // sequence of turns whatever happens (an expired wait only skips the
 // arithmetic), so that the sweep always comes to its end.
-template <int NP, bool DOWN, typename X>
+// LONG: rows of more than 16 entries.  What they have beyond their record stays in the
+// ring until the group is done and is read there, after the slice before is stored;
+// three records are held instead of four, so that nothing spills.  us per application,
+// 64^3 mixed: 20 entries 283, 30 entries 611 (one warp walking such levels slice by
+// slice 701 and 1178; chunks taken by four warps in turn, before the streams, 487 and
+// 900); 80^3 in 8 blocks (vectors in global memory), 20 entries 4.30 ms (5.89, 4.65).
+template <int NP, bool LONG, bool DOWN, typename X>
 __device__ __forceinline__ void consume_groups(ItemWalk &W, const X &x, int warp, int lane, int &g, int end, bool &ok) {
     constexpr int LP = NP < kLatePairs ? NP : kLatePairs;
     const int nw = (warp + 1) % 4;
@@ -110,13 +157,20 @@ __device__ __forceinline__ void consume_groups(ItemWalk &W, const X &x, int warp
             give_turn(kFinal + nw);
             continue;
         }
-        RowF32<NP> R[4];
-        const int4 d = lds<int4>(p);            // rows - 1 and (high half) place of every slice
-        fetch_f32(p + (d.x >> 16), d.x & 0xffff, lane, R[0]);
-        fetch_f32(p + (d.y >> 16), d.y & 0xffff, lane, R[1]);
-        fetch_f32(p + (d.z >> 16), d.z & 0xffff, lane, R[2]);
-        fetch_f32(p + (d.w >> 16), d.w & 0xffff, lane, R[3]);
-        W.next(lane);
+        constexpr int kHeld = LONG ? 3 : 4;     // records in registers
+        RowF32<NP> R[kHeld];
+        const int4 dx = lds<int4>(p);           // rows - 1 and (high half) place of every slice
+        const int d[4] = {dx.x, dx.y, dx.z, dx.w};
+#pragma unroll
+        for (int s = 0; s < (LONG ? 2 : 4); ++s) fetch_f32(p + (d[s] >> 16), d[s] & 0xffff, lane, R[s]);
+        int4 rx = make_int4(0, 0, 0, 0);        // LONG: where the rests are
+        RestF32 rest[2];
+        if constexpr (LONG) {
+            rx = lds<int4>(p + kItemHeader);
+            rest[0].fetch(p, rx.x, min(lane, d[0] & 0xffff));
+        } else {
+            W.next(lane);
+        }
         float xv[2][2 * NP], self[2];
         await_turn(kEarly + warp);
         gather_f32<0, NP - LP>(R[0], x, xv[0]);
@@ -124,47 +178,26 @@ __device__ __forceinline__ void consume_groups(ItemWalk &W, const X &x, int warp
         await_turn(kFinal + warp);
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-            gather_f32<NP - LP, NP>(R[s], x, xv[s & 1]);
+            const RowF32<NP> &now = R[s % kHeld], &next = R[(s + 1) % kHeld];
+            gather_f32<NP - LP, NP>(now, x, xv[s & 1]);
             if (s < 3) {
-                gather_f32<0, NP - LP>(R[s + 1], x, xv[(s + 1) & 1]);
-                self[(s + 1) & 1] = x.load(R[s + 1].row);
+                gather_f32<0, NP - LP>(next, x, xv[(s + 1) & 1]);
+                self[(s + 1) & 1] = x.load(next.row);
             }
-            x.store(R[s].row, row_f32<NP, DOWN>(R[s], xv[s & 1], self[s & 1]));
+            const int desc[4] = {rx.x, rx.y, rx.z, rx.w};
+            if constexpr (LONG) {
+                if (s < 2) fetch_f32(p + (d[s + 2] >> 16), d[s + 2] & 0xffff, lane, R[(s + 2) % kHeld]);
+                if (s < 3) rest[(s + 1) & 1].fetch(p, desc[s + 1], min(lane, d[s + 1] & 0xffff));
+            }
+            x.store(now.row, row_f32<NP, DOWN>(now, xv[s & 1], self[s & 1], [&](float a) {
+                        if constexpr (LONG) return rest[s & 1].add(desc[s], x, a);
+                        else return a;
+                    }));
             __syncwarp();
             if (s == 2) give_turn(kEarly + nw);
         }
         give_turn(kFinal + nw);
-    }
-}
-
-// Levels with longer rows: one warp, slice by slice.
-template <typename X>
-__device__ __forceinline__ void consume_long_rows(ItemWalk &W, const X &x, int lane, int nitem) {
-    constexpr int NP = 8;
-    for (int g = 0; g < nitem; ++g) {
-        uint32_t p = W.item();
-        if (!p) return;
-        const int4 h = lds<int4>(p);
-        p += kItemHeader;
-        RowF32<NP> R;
-        fetch_f32(p, h.x, lane, R);
-        float xv[2 * NP], a0 = 0, a1 = 0;
-        gather_f32<0, NP>(R, x, xv);
-        const float self = x.load(R.row);
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            a0 += __int_as_float(R.e[i].y) * xv[2 * i];
-            a1 += __int_as_float(R.e[i].w) * xv[2 * i + 1];
-        }
-        p += ((8 * h.x + 23) & ~15) + row_bytes(NP) * (h.x + 1) + 8 * min(lane, h.x);
-        for (int i = 0; i < h.z; ++i, p += 8 * (h.x + 1)) {
-            const int2 e = lds<int2>(p);
-            if (e.x >= 0) a0 += __int_as_float(e.y) * x.load(e.x);
-        }
-        // lanes past the last row hold it too: they must not store, another of them
-        // may still have its x_i to read
-        if (lane <= h.x) x.store(R.row, fmaf(self, R.dinv, sum_rn(a0, a1)));
-        W.next(lane);
+        if constexpr (LONG) W.next(lane);
     }
 }
 
@@ -351,6 +384,7 @@ k_trsv(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restric
             mbar_init(&H->empty[s], OneLaneRows<VT>::value ? 1 : 4);
         }
         H->abort_flag = 0;
+        H->no_entry = 0.f;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -425,8 +459,9 @@ k_trsv(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restric
         const BlockVec<VT, SMEM> x(xs);
         ItemWalk W(lv.S, H, ring, OneLaneRows<VT>::value ? warp : warp / 4);
         if constexpr (!OneLaneRows<VT>::value) consume_lanes<NP, NS, VT>(W, x, warp, lane, i1 - i0, lv.S.split[b]);
-        else if constexpr (NP == kLongRows) consume_long_rows(W, x, lane, i1 - i0);
         else if (i1 > i0) {
+            constexpr bool kLong = NP == kLongRows;
+            constexpr int kPairs = kLong ? 8 : NP;
             const int ng = i1 - i0, nl = lv.S.split[b];
             int g = warp;
             bool ok = true;
@@ -434,8 +469,8 @@ k_trsv(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restric
                 give_turn(kEarly);
                 give_turn(kFinal);
             }
-            consume_groups<NP, false>(W, x, warp, lane, g, nl, ok);
-            consume_groups<NP, true>(W, x, warp, lane, g, ng, ok);
+            consume_groups<kPairs, kLong, false>(W, x, warp, lane, g, nl, ok);
+            consume_groups<kPairs, kLong, true>(W, x, warp, lane, g, ng, ok);
             if (warp == ng % 4) {               // and the last group's
                 await_turn(kEarly + warp);
                 await_turn(kFinal + warp);
@@ -474,7 +509,7 @@ void with_trsv(int np, int ns, Fn f) {
             case 3: return call(i3, i4);
             case 5: return call(i5, i4);
             case 8: return call(i8, i4);
-            default: return call(il, i1);
+            default: return call(il, i4);
         }
     } else {
         auto either = [&](auto n) {
@@ -494,7 +529,9 @@ void with_trsv(int np, int ns, Fn f) {
 
 // Entries per record (FP32: pairs of entries, FP64: entries of each of four lanes) by
 // the level's longest row: every entry of a record is gathered and summed, so the
-// sizes step with the chains' lengths; rows past the largest record walk the rest.
+// sizes step with the chains' lengths; rows past the largest record read their rest
+// from the staged item, at 283 us per 64^3 mixed application with 20 entries against
+// 222 with 16.
 int trsv_record(bool one_lane, int longest) {
     if (one_lane) return longest <= 2 ? 1 : longest <= 6 ? 3 : longest <= 10 ? 5 : longest <= 16 ? 8 : kLongRows;
     return longest <= 4 ? 1 : longest <= 8 ? 2 : longest <= 12 ? 3 : 4;

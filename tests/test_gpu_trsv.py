@@ -173,3 +173,55 @@ def test_batched_large_blocks_against_plain_solves(name, nsys, per_cta):
     for s, q in ((0, 0), (0, 7), (1, 3), (nsys - 1, 0), (nsys - 1, 7)):
         ref = _solved(blocks, sizes, r[s, q])
         assert np.max(np.abs(z[s, q] - ref)) <= 3e-5 * np.max(np.abs(ref)), (s, q)
+
+
+# One row longer than a record must not change a whole level's schedule.  The variant
+# for such levels adds a test to the work on a slice, and for the slice of that row
+# one more read and gather (about 60 of 200 cycles): half as long again is the bound,
+# where one warp walking the level alone took two to three times as long.
+def test_one_long_row_costs_little():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_03224_gb300 import Gemslr
+    CASES["long_row"] = ([3000, 3000], 16, 300, False)
+    _, blocks, sizes, A, part, fac = _system("long_row", False)
+    times = []
+    for longer in (False, True):
+        if longer:
+            L = fac["levels"][0]["L"].tolil()
+            free = sorted(set(range(2000, 2990)) - set(L.rows[2990]))
+            for c in free[:: len(free) // 17][: 17 - len(L.rows[2990])]:
+                L[2990, c] = 1e-3
+            fac["levels"][0]["L"] = L.tocsr()
+            assert np.diff(fac["levels"][0]["L"].indptr).max() == 17
+        G = Gemslr.from_factors(A, part, fac, precision="mixed")
+        r = torch.rand(A.n, dtype=torch.float64, device="cuda")
+        best = float("inf")
+        for _ in range(8):
+            start, end = torch.cuda.Event(True), torch.cuda.Event(True)
+            start.record()
+            for _ in range(20):
+                G.apply(r)
+            end.record()
+            end.synchronize()
+            best = min(best, start.elapsed_time(end))
+        times.append(best)
+    assert times[1] <= 1.5 * times[0], times
+
+
+# Rests so long that few rows, or one, fill a group's item.  The bound of the module's
+# note for m = 300: 8 (m + 3) eps = 1.45e-4.
+@pytest.mark.parametrize("rows,chain", [(900, False), (900, True)])
+def test_rows_of_hundreds_of_entries(rows, chain):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_03224_gb300 import Gemslr
+    CASES["hundreds"] = ([rows, 350], 300, 800, chain)
+    rng, blocks, sizes, A, part, fac = _system("hundreds", False)
+    G = Gemslr.from_factors(A, part, fac, precision="mixed")
+    r = rng.uniform(-1, 1, A.n)
+    z = G.apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    ref = _solved(blocks, sizes, r)
+    assert np.max(np.abs(z - ref)) <= 1.6e-4 * np.max(np.abs(ref)), np.max(np.abs(z - ref))
