@@ -378,14 +378,14 @@ k_trsv(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restric
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char *ring = smem + kHead + (SMEM ? ring_offset : 0);
     const int i0 = lv.S.blk_item[b], i1 = lv.S.blk_item[b + 1];
+    if ((int)threadIdx.x < lv.S.slots) {        // a thread per slot: one after another, 64 slots take a microsecond
+        mbar_init(&H->full[threadIdx.x], 1);
+        mbar_init(&H->empty[threadIdx.x], OneLaneRows<VT>::value ? 1 : 4);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < lv.S.slots; ++s) {
-            mbar_init(&H->full[s], 1);
-            mbar_init(&H->empty[s], OneLaneRows<VT>::value ? 1 : 4);
-        }
         H->abort_flag = 0;
         H->no_entry = 0.f;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     if (warp == kWarps) {                       // producer
