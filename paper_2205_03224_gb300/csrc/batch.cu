@@ -158,6 +158,9 @@ bool build_streams(gemslr_batch_ctx *B, int l, bool last, const std::vector<int3
     sh.np = trsv_record(true, (int)longest);
     sh.consumers = kBatchSets;
     if (sh.np == kLongRows) return false;
+    const size_t optin = (size_t)dev_smem_optin();
+    for (int32_t nr : blk_nr)
+        if (bstream_smem(nr, kBatchRhs / 2, StreamView{}) > optin) return false;
     int64_t lb = 0, ub = 0;
     for (int s = 0; s < B->nsys; ++s)
         append_batch_stream(level(s).L, level(s).U, level(s).bp, kBatchSliceRows, kBatchItemBytes, sh, lb, ub);
@@ -169,7 +172,6 @@ bool build_streams(gemslr_batch_ctx *B, int l, bool last, const std::vector<int3
     int dev = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    const size_t optin = (size_t)dev_smem_optin();
     struct Unit { int32_t blk, rhs0, rpc, fit, items; };
     std::vector<Unit> all;
     for (size_t b = 0; b < blk_nr.size(); ++b) {

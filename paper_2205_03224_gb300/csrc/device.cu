@@ -316,30 +316,30 @@ struct EntryF32 { int32_t col; float v; };
 
 // FP32 row i into its record of np pairs: pair p at slot(p), entries from 16 on to rest.
 template <typename Slot>
-void put_row_f32(const Csr &T, int64_t r0, int64_t i, bool upper, EntryF32 *rec, Slot slot, EntryF32 *rest) {
+void put_row_f32(const Csr &T, int64_t r0, int64_t i, bool upper, int64_t unit, EntryF32 *rec, Slot slot, EntryF32 *rest) {
     const int64_t pdiag = upper ? diagonal(T, i) : -1;
     int64_t e = 0;
     for (int64_t p = T.rp[i]; p < T.rp[i + 1]; ++p) {
         if (T.ci[p] == i) continue;
-        const EntryF32 en{(int32_t)((T.ci[p] - r0) * 4), stored_entry<float>(T, p, pdiag)};
+        const EntryF32 en{vector_place(T.ci[p] - r0, unit), stored_entry<float>(T, p, pdiag)};
         if (e < 16) rec[2 * slot(e / 2) + e % 2] = en;
         else rest[e - 16] = en;
         ++e;
     }
 }
-EntryF32 row_head_f32(const Csr &T, int64_t r0, int64_t i, bool upper) {
-    return {(int32_t)((i - r0) * 4), upper ? inv_entry<float>(T, diagonal(T, i)) : 1.f};
+EntryF32 row_head_f32(const Csr &T, int64_t r0, int64_t i, bool upper, int64_t unit) {
+    return {vector_place(i - r0, unit), upper ? inv_entry<float>(T, diagonal(T, i)) : 1.f};
 }
 
 // FP32: rows to their heads and records of np pairs, entries from 16 on to their rests.
 void put_rows_f32(const Csr &T, int64_t r0, const Waves &W, bool upper, const int64_t *rows, int64_t n, int np,
-                  unsigned char *p, unsigned char *rest, size_t rest_bytes) {
+                  int64_t unit, unsigned char *p, unsigned char *rest, size_t rest_bytes) {
     EntryF32 *head = reinterpret_cast<EntryF32 *>(p);
     unsigned char *recs = p + pad16((size_t)(8 * n));
     for (int64_t t = 0; t < n; ++t) {
         const int64_t i = rows[t], shift = np - (std::min<int64_t>(16, W.len[i - r0]) + 1) / 2;
-        head[t] = row_head_f32(T, r0, i, upper);
-        put_row_f32(T, r0, i, upper, reinterpret_cast<EntryF32 *>(recs + row_bytes(np) * t),
+        head[t] = row_head_f32(T, r0, i, upper, unit);
+        put_row_f32(T, r0, i, upper, unit, reinterpret_cast<EntryF32 *>(recs + row_bytes(np) * t),
                     [&](int64_t pr) { return upper ? np - 1 - pr : pr + shift; },
                     reinterpret_cast<EntryF32 *>(rest + rest_bytes * t));
     }
@@ -422,7 +422,7 @@ void append_groups(const Csr &T, int64_t r0, const Waves &W, bool upper, StreamH
                 for (size_t e = 0; e < c.rests() / sizeof(EntryF32); ++e) reinterpret_cast<EntryF32 *>(rest)[e] = {kNoEntry, 0.f};
             }
             if (k < 0) *reinterpret_cast<EntryF32 *>(p + off) = {kNoRow, 1.f};
-            else put_rows_f32(T, r0, W, upper, c.rows, c.n, np, p + off, rest, rest_bytes((int)c.quads));
+            else put_rows_f32(T, r0, W, upper, c.rows, c.n, np, out.unit, p + off, rest, rest_bytes((int)c.quads));
             off += bytes(k);
         }
     }
@@ -445,7 +445,7 @@ struct LaneSlices {
 };
 
 template <typename VT>
-void append_lanes(const Csr &T, int64_t r0, const Waves &W, bool upper, int np, LaneSlices &out) {
+void append_lanes(const Csr &T, int64_t r0, const Waves &W, bool upper, int np, int64_t unit, LaneSlices &out) {
     const size_t lb = lane_bytes<VT>(np), tb = pad16(sizeof(VT) + 4);
     auto bytes = [&](int64_t n, int64_t m) {
         return kItemHeader + (size_t)(4 * n) * (lb + (size_t)std::max<int64_t>(0, (m + 3) / 4 - 4) * tb);
@@ -461,11 +461,11 @@ void append_lanes(const Csr &T, int64_t r0, const Waves &W, bool upper, int np, 
                 const int64_t i = s.rows[at + t], pdiag = upper ? diagonal(T, i) : -1;
                 auto put = [&](unsigned char *rv, unsigned char *rc, int64_t col, VT v) {
                     *reinterpret_cast<VT *>(rv) = v;
-                    *reinterpret_cast<int32_t *>(rc) = (int32_t)((col - r0) * (int64_t)sizeof(VT));
+                    *reinterpret_cast<int32_t *>(rc) = vector_place(col - r0, unit);
                 };
                 for (int64_t q = 0; q < 4; ++q)
                     *reinterpret_cast<int32_t *>(p + lb * (4 * t + q) + np * (sizeof(VT) + 4)) =
-                        (int32_t)((i - r0) * (int64_t)sizeof(VT));
+                        vector_place(i - r0, unit);
                 int64_t e = 0;
                 for (int64_t pp = T.rp[i]; pp < T.rp[i + 1]; ++pp) {
                     if (T.ci[pp] == i) continue;
@@ -535,7 +535,7 @@ int32_t pack_lanes(LaneSlices &s, size_t item_bytes, StreamHost &out) {
 
 // Slices of one factor in the batched layout (batch.cuh).
 void append_batch_rows(const Csr &T, int64_t r0, const Waves &W, bool upper, int np, int max_rows, LaneSlices &out) {
-    auto place = [&](int64_t i) { return (int32_t)((i - r0 + 1) * 16); };
+    auto place = [&](int64_t i) { return vector_place(i - r0 + 1, 16); };
     for (const SliceRows &s : cut_slices<float>(W, r0, upper, max_rows)) {
         unsigned char *p = out.add(kItemHeader + pad16((size_t)(8 * s.n)) + (size_t)(row_bytes(np) * s.n), s.n, 0,
                                    s.sync ? kSync : 0);
@@ -608,9 +608,9 @@ void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, St
             append_groups(U, r0, wu[b], true, out);
         } else {
             LaneSlices s;
-            append_lanes<VT>(L, r0, wl[b], false, out.np, s);
+            append_lanes<VT>(L, r0, wl[b], false, out.np, out.unit, s);
             append_scaling<VT>(U, r0, bp[b + 1] - r0, s);
-            append_lanes<VT>(U, r0, wu[b], true, out.np, s);
+            append_lanes<VT>(U, r0, wu[b], true, out.np, out.unit, s);
             out.split.push_back(pack_lanes(s, kLaneItemBytes, out));
         }
         out.blk_item.push_back((int32_t)(out.off.size() - 1));
@@ -639,6 +639,7 @@ void upload_level(const HostLevel &hl, int64_t n, bool schur, Arena &a, DevLevel
     for (size_t b = 0; b + 1 < hl.bp.size(); ++b) maxrows = std::max(maxrows, hl.bp[b + 1] - hl.bp[b]);
     d.smem_rows = (kRingBytes + maxrows * (int64_t)sizeof(VT) <= smem_limit) ? (int)maxrows : 0;
     StreamHost sh;
+    sh.unit = place_unit<VT>(d.smem_rows > 0);
     build_stream<VT>(hl.L, hl.U, hl.bp, sh);
     v.S.data = a.upload(sh.data);
     v.S.off = a.upload(sh.off);

@@ -135,6 +135,7 @@ struct StreamHost {                    // single-system substitutions (see Strea
     std::vector<int64_t> off{0};
     std::vector<int32_t> blk_item{0}, split;
     int np = 0, consumers = 1;
+    int64_t unit = 1;                  // place_unit of the level
     int slot_bytes = 0;                // largest item
     int maxwf_L = 0, maxwf_U = 0;      // wavefronts (largest over the blocks)
 };
@@ -144,7 +145,7 @@ struct StreamHost {                    // single-system substitutions (see Strea
 void append_batch_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, int max_rows, size_t item_bytes,
                          StreamHost &out, int64_t &l_bytes, int64_t &u_bytes);
 template <typename VT>
-void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, StreamHost &out);
+void build_stream(const Csr &L, const Csr &U, const std::vector<int64_t> &bp, StreamHost &out);   // out.unit set
 
 // ---- device memory arena ------------------------------------------------------------
 class Arena {

@@ -27,6 +27,12 @@ struct Error {
 };
 [[noreturn]] void fail(gemslr_status st, const std::string &msg);
 
+// Place of a block's row in the factor streams: its number (unit 1) or byte offset, an int32.
+inline int32_t vector_place(int64_t row, int64_t unit) {
+    if (row > INT32_MAX / unit) fail(GEMSLR_ERR_UNSUPPORTED, "a block has more rows than the substitutions can address");
+    return (int32_t)(row * unit);
+}
+
 // u in [0, 1) from splitmix64(seed): the first `count` outputs' top 53 bits
 // (the seeded start vectors and random blocks of the set-up; setup.cpp).
 std::vector<double> splitmix_uniform01(uint64_t seed, int64_t count);

@@ -22,7 +22,8 @@ constexpr int kMaxCols = 160;     // Krylov columns per Gram-Schmidt pass (m + 1
 // multiple of consumers, so that a slot has one reader).
 // Values are -t_ij (L) and -u_ij/u_ii (U), formed in FP64 and rounded once, so
 // that a row is x_i = x_i d_i + sum_j v_ij x_j with d_i = 1 (L) or 1/u_ii (U);
-// rows and columns are byte offsets into the block's vector.
+// rows and columns are places in the block's vector, place_unit per row: byte offsets,
+// or row numbers (FP64 and complex vectors in global memory).
 //
 // FP32: x_i = fma(x_i, d_i, a0 + a1), a0 the sum of the even entries and of
 // those from 16 on, a1 that of the odd ones below 16, in order; one lane per row,
@@ -65,7 +66,7 @@ template <typename VT> constexpr int kLaneRows = sizeof(VT) == 8 ? 32 : 16;   //
 constexpr int kMaxItemBytes = 16192;            // head and a slot for each of four consumers within kRingBytes
 constexpr int kItemDepth = 16;                  // most slots per consumer
 constexpr int kLatePairs = 3;
-constexpr int kNoRow = -4, kNoEntry = -8;      // places in the StreamHead
+constexpr int kNoRow = -4, kNoEntry = -8;      // byte offsets of words of the StreamHead
 constexpr int kLaneItemBytes = 8192;            // FP64: slices of a consumer are joined into items of about this size
 constexpr int kLongRows = 16;
 constexpr int kRestQuads = 16;
@@ -74,6 +75,8 @@ enum { kSync = 1 };
 enum { kLaneShift = 4, kLane1 = 0, kLane2, kLane4, kLaneFull, kLaneLong, kLaneScale };
 template <typename VT> struct OneLaneRows { static constexpr bool value = false; };
 template <> struct OneLaneRows<float> { static constexpr bool value = true; };
+template <typename VT>
+__host__ __device__ constexpr int64_t place_unit(bool smem) { return smem || OneLaneRows<VT>::value ? sizeof(VT) : 1; }
 __host__ __device__ constexpr int odd16(int bytes) { return (((bytes + 15) / 16) | 1) * 16; }
 __host__ __device__ constexpr int row_bytes(int np) { return odd16(16 * np); }
 __host__ __device__ constexpr int rest_bytes(int quads) { return odd16(32 * quads); }

@@ -34,8 +34,8 @@ __device__ __forceinline__ zc mul_rn(zc a, zc b) {
 }
 
 // ---- FP32 rows -----------------------------------------------------------------------
-// A row in registers: byte offset of x_i, d_i, and NP pairs of entries (byte
-// offset of x_j, value).
+// A row in registers: place of x_i, d_i, and NP pairs of entries (place of x_j,
+// value).
 template <int NP>
 struct RowF32 {
     int row;
@@ -202,7 +202,7 @@ __device__ __forceinline__ void consume_groups(ItemWalk &W, const X &x, int warp
 }
 
 // ---- FP64 and complex: four lanes per row ----------------------------------------------
-// A lane's share of a row in registers: its first KQ entries and the byte offset of x_i.
+// A lane's share of a row in registers: its first KQ entries and the place of x_i.
 template <typename VT, int KQ>
 struct RowF64 {
     static constexpr int kV = (int)sizeof(VT) / 4, kUsed = (KQ * ((int)sizeof(VT) + 4) + 4 + 15) / 16;
@@ -336,7 +336,7 @@ __device__ __forceinline__ void consume_lanes(ItemWalk &W, const X &x, int warp,
                 // rows z .. z + h.x of x times their 1 / u_ii: dense, every lane busy
                 for (int k = h.w >> 24; k > 0; --k, --nsync) wavefront_end<NT>(1);
                 for (int i = 32 * (warp % 4) + lane; i <= h.x; i += 128) {
-                    const int a = (h.z + i) * (int)sizeof(VT);
+                    const int a = x.place(h.z + i);
                     x.store(a, mul_rn(x.load(a), lds<VT>(p + kItemHeader + i * (int)sizeof(VT))));
                 }
                 wavefront_end<NT>(h.w & kSync);
