@@ -225,3 +225,27 @@ def test_rows_of_hundreds_of_entries(rows, chain):
     z = G.apply(torch.from_numpy(r).cuda()).cpu().numpy()
     ref = _solved(blocks, sizes, r)
     assert np.max(np.abs(z - ref)) <= 1.6e-4 * np.max(np.abs(ref)), np.max(np.abs(z - ref))
+
+
+# Streamed batched levels whose blocks hold four right-hand sides at a time, beside
+# blocks that hold all eight.  The levels that are not streamed would take four here
+# only in one wave (152 CTAs), and these blocks are more than that: so four is the
+# streamed split.
+@pytest.mark.parametrize("nrhs", [1, 5, 8])
+@pytest.mark.parametrize("most", [3, 10, 16])
+def test_batched_streams_of_four_right_hand_sides(most, nrhs):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_03224_gb300 import GemslrBatch
+    CASES["four"] = ([9000, 8500, 300], most, 500, False)
+    _, blocks, sizes, A, part, fac = _system("four", False)
+    nsys = 40
+    B = GemslrBatch.from_factors([A] * nsys, [part] * nsys, [fac] * nsys)
+    assert B.stats()["rhs_per_cta"] == 4
+    rng = np.random.default_rng(nrhs)
+    r = rng.uniform(-1, 1, (nsys, nrhs, A.n))
+    z = B.apply(torch.from_numpy(r.ravel()).cuda(), nrhs).cpu().numpy().reshape(r.shape)
+    for s, q in {(0, 0), (17, nrhs // 2), (nsys - 1, nrhs - 1)}:
+        ref = _solved(blocks, sizes, r[s, q])
+        assert np.max(np.abs(z[s, q] - ref)) <= 3e-5 * np.max(np.abs(ref)), (s, q)
