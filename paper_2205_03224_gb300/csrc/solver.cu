@@ -127,9 +127,12 @@ void ensure_krylov(gemslr_ctx *h, int m) {
         h->r = (double *)h->arena.alloc(8 * n);
         h->w = (double *)h->arena.alloc(8 * n);
         h->red_grid = sm_count();                 // one CTA per SM: few partials for the finisher
-        // FGMRES on small systems: a CTA per 256 rows, fewer partials for the last CTA
-        // (n = 1,024: 4 per column instead of 152; w = A z and its reduction 22.0 ->
-        // 19.9 us, the solve's 35 iterations 2679 -> 2571 us)
+        // FGMRES on small systems: a CTA per 256 rows, fewer partials for the last CTA to
+        // add and fewer hand-overs.  ms per solve with 128 rows / 256 / a CTA per SM: n = 256
+        // 1.17 / 1.19 / 1.25, 1,024 1.95 / 1.99 / 2.08, 4,096 2.46 / 2.49 / 2.54, 6,724 7.09 /
+        // 7.20 / 7.40, 14,400 12.60 / 12.70 / 12.89, 19,881 17.23 / 17.07 / 17.23, 34,969 29.99 /
+        // 29.96 / 29.99: above 15,000 fewer rows are too little work per CTA, below they gain
+        // up to 2%
         h->solve_grid = (int)std::min<int64_t>(h->red_grid, (n + kReduceThreads - 1) / kReduceThreads);
         h->partial = (double *)h->arena.alloc(8 * (size_t)h->red_grid * (2 * kMaxCols + 4));
         h->counter = (unsigned *)h->arena.alloc(16);
