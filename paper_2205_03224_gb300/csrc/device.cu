@@ -647,9 +647,20 @@ void upload_level(const HostLevel &hl, int64_t n, bool schur, Arena &a, DevLevel
     v.S.split = a.upload(sh.split);
     v.S.np = sh.np;
     v.S.consumers = sh.consumers;
+    // More blocks than SMs: a ring that leaves room for up to three CTAs on an SM, in FP32
+    // without the four warps that only help (their registers are another CTA's).  us per
+    // application with a CTA per SM / now: 96^3 in 1,024 blocks mixed 370 / 204, FP64 1315 /
+    // 1146; 64^3 in 256 mixed 142 / 90, FP64 483 / 392, complex 975 / 913.
+    int dev = 0, sms = 1, per_sm = 0;
+    GEMSLR_CUDA(cudaGetDevice(&dev));
+    GEMSLR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    GEMSLR_CUDA(cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    const int64_t share = d.smem_rows ? std::min<int64_t>(3, (v.nblk + sms - 1) / sms) : 1;
+    v.S.variant = !OneLaneRows<VT>::value ? sh.consumers : share > 1 ? 4 : 8;
     // the ring: up to kItemDepth slots per consumer, in twice kRingData where the
     // vector leaves that much (more bytes in flight), at least one
-    const int64_t room = (d.smem_rows ? smem_limit - (int64_t)pad16(d.smem_rows * sizeof(VT)) : (int64_t)kRingBytes) -
+    const int64_t limit = std::min<int64_t>(smem_limit, per_sm / std::max<int64_t>(1, share) - 1024);
+    const int64_t room = (d.smem_rows ? limit - (int64_t)pad16(d.smem_rows * sizeof(VT)) : (int64_t)kRingBytes) -
                          (int64_t)sizeof(StreamHead);
     v.S.slot_bytes = std::max(sh.slot_bytes, 128);
     const int64_t depth = std::min<int64_t>(room, 2 * kRingData) / ((int64_t)v.S.slot_bytes * sh.consumers);

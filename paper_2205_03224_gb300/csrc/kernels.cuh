@@ -100,6 +100,7 @@ struct StreamView {
     int32_t np;                // pairs per row record (FP32), entries per lane record (FP64)
     int32_t consumers;         // FP32: 4; FP64: 2 or 4
     int32_t slots, slot_bytes; // the ring
+    int32_t variant;           // FP32: compute warps of a CTA, 8 or 4; FP64: consumers
 };
 
 // ---- chunks of the batched substitutions --------------------------------------------

@@ -348,17 +348,18 @@ __device__ __forceinline__ void consume_lanes(ItemWalk &W, const X &x, int warp,
     for (; nsync > 0; --nsync) wavefront_end<NT>(1);
 }
 
-// Warps that form the right-hand side and store the result: those that walk
-// the stream and, when they are few, others that only help with this.
+// Warps that form the right-hand side and store the result: those that walk the
+// stream and, when they are few, others that only help with this (FP32: NS is their
+// number, 8 or the four that walk).
 template <typename VT>
 __host__ __device__ constexpr int compute_warps(int ns) {
-    return OneLaneRows<VT>::value || ns < 4 ? 8 : 4 * ns;
+    return OneLaneRows<VT>::value ? ns : ns < 4 ? 8 : 4 * ns;
 }
 
 // MODE 0: right-hand side from `in` (FP64 user vector) or `work`; result in work.
 // MODE 1: right-hand side F y2 (gathered from work's tail); work[rows] -= result.
 // The last warp is the producer; the others form the right-hand side and store
-// the result together, the first NS (FP32) or the NS sets of four of them walk
+// the result together, the first four (FP32) or the NS sets of four of them walk
 // the stream.
 template <typename VT, typename WT, int MODE, bool SMEM, int NP, int NS>
 __global__ void __launch_bounds__(32 * (compute_warps<VT>(NS) + 1))
@@ -366,7 +367,7 @@ k_trsv(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restric
        IoT<VT> *__restrict__ out_final, VT *__restrict__ scratch, const PendingLowRank<VT, WT> pl, int ring_offset) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int kWarps = compute_warps<VT>(NS), NC = 32 * kWarps;
-    constexpr int kWalkers = OneLaneRows<VT>::value ? NS : 4 * NS;
+    constexpr int kWalkers = OneLaneRows<VT>::value ? 4 : 4 * NS;
     StreamHead *H = reinterpret_cast<StreamHead *>(smem);
     constexpr int kHead = sizeof(StreamHead);
     VT *xs_smem = reinterpret_cast<VT *>(smem + kHead);
@@ -490,7 +491,7 @@ k_trsv(const LevelView<VT, WT> lv, const IoT<VT> *__restrict__ in, VT *__restric
     }
 }
 
-// Calls f with the kernel instantiation of a level's variant (StreamView::np, consumers).
+// Calls f with the kernel instantiation of a level's variant (StreamView::np, variant).
 template <typename VT, typename WT, int MODE, bool SMEM, typename Fn>
 void with_trsv(int np, int ns, Fn f) {
     auto call = [&](auto n, auto c) {
@@ -504,12 +505,18 @@ void with_trsv(int np, int ns, Fn f) {
     constexpr std::integral_constant<int, 8> i8;
     constexpr std::integral_constant<int, kLongRows> il;
     if constexpr (OneLaneRows<VT>::value) {
+        auto either = [&](auto n) {
+            if constexpr (SMEM) {
+                if (ns == 4) return call(n, i4);
+            }
+            call(n, i8);
+        };
         switch (np) {
-            case 1: return call(i1, i4);
-            case 3: return call(i3, i4);
-            case 5: return call(i5, i4);
-            case 8: return call(i8, i4);
-            default: return call(il, i4);
+            case 1: return either(i1);
+            case 3: return either(i3);
+            case 5: return either(i5);
+            case 8: return either(i8);
+            default: return either(il);
         }
     } else {
         auto either = [&](auto n) {
@@ -553,11 +560,11 @@ void launch_trsv(const LevelView<VT, WT> &lv, int mode, int smem_rows, const IoT
         kernel<<<lv.nblk, 32 * (warps + 1), bytes, st>>>(lv, in, work, out_final, scratch, pl, ring_offset);
     };
     if (smem_rows > 0) {
-        if (mode == 0) with_trsv<VT, WT, 0, true>(lv.S.np, lv.S.consumers, go);
-        else with_trsv<VT, WT, 1, true>(lv.S.np, lv.S.consumers, go);
+        if (mode == 0) with_trsv<VT, WT, 0, true>(lv.S.np, lv.S.variant, go);
+        else with_trsv<VT, WT, 1, true>(lv.S.np, lv.S.variant, go);
     } else {
-        if (mode == 0) with_trsv<VT, WT, 0, false>(lv.S.np, lv.S.consumers, go);
-        else with_trsv<VT, WT, 1, false>(lv.S.np, lv.S.consumers, go);
+        if (mode == 0) with_trsv<VT, WT, 0, false>(lv.S.np, lv.S.variant, go);
+        else with_trsv<VT, WT, 1, false>(lv.S.np, lv.S.variant, go);
     }
     count_launch();
 }
@@ -575,7 +582,7 @@ void set_trsv_smem_limit(int bytes) {
     for (int longest : {1, 5, 9, 16, 17})
         for (bool first : {true, false}) {
             const int np = trsv_record(one, longest);
-            const int ns = trsv_sets(first ? 0.0 : 1e9);
+            const int ns = one ? (first ? 4 : 8) : trsv_sets(first ? 0.0 : 1e9);
             with_trsv<VT, WT, 0, true>(np, ns, in_smem);
             with_trsv<VT, WT, 1, true>(np, ns, in_smem);
             with_trsv<VT, WT, 0, false>(np, ns, in_global);

@@ -249,3 +249,23 @@ def test_batched_streams_of_four_right_hand_sides(most, nrhs):
     for s, q in {(0, 0), (17, nrhs // 2), (nsys - 1, nrhs - 1)}:
         ref = _solved(blocks, sizes, r[s, q])
         assert np.max(np.abs(z[s, q] - ref)) <= 3e-5 * np.max(np.abs(ref)), (s, q)
+
+
+# More blocks than SMs (152): CTAs share an SM, in FP32 with the four walking warps
+# only; every record size, and blocks of one row among them.
+@pytest.mark.parametrize("kind", ["fp64", "mixed", "complex"])
+@pytest.mark.parametrize("most", [1, 6, 10, 16, 20])
+def test_more_blocks_than_sms_against_plain_solves(most, kind):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_03224_gb300 import Gemslr
+    cplx = kind == "complex"
+    CASES["many"] = ([61, 1, 40, 90] * 80, most, 30, False)
+    rng, blocks, sizes, A, part, fac = _system("many", cplx)
+    G = Gemslr.from_factors(A, part, fac, precision="mixed" if kind == "mixed" else "fp64")
+    r = rng.uniform(-1, 1, A.n) + (1j * rng.uniform(-1, 1, A.n) if cplx else 0)
+    z = G.apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    ref = _solved(blocks, sizes, r)
+    tol = 3e-5 if kind == "mixed" else 1e-13
+    assert np.max(np.abs(z - ref)) <= tol * np.max(np.abs(ref)), np.max(np.abs(z - ref))
