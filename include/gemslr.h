@@ -357,8 +357,8 @@ void gemslr_destroy(gemslr_handle h);
 /*
  * Batched solve phase: many independent systems (each with its own CSR,
  * multilevel partition and setup, Alg. 1) handled together with up to
- * GEMSLR_BATCH_RHS right-hand sides each.  Every stage of M^{-1} (Alg. 2) is
- * one launch over all systems; FGMRES runs for every (system, rhs) pair in
+ * GEMSLR_BATCH_RHS right-hand sides each.  Every stage of M^{-1} (Alg. 2) covers
+ * all systems; FGMRES runs for every (system, rhs) pair in
  * lock step, the whole solve being one CUDA graph (GEMSLR_SOLVE_GRAPH=0: a
  * host loop, as for gemslr_fgmres_solve); a system whose pairs have all
  * stopped is skipped by the rest of the cycle's steps.  The preconditioner is
@@ -383,8 +383,9 @@ void gemslr_destroy(gemslr_handle h);
  * block rows (all systems), bytes of its stored L slices and of its U slices,
  * and the nonzeros of its F (what one down and one up sweep of that level
  * must read).
- * An application launches independent blocks on streams of the handle, forked
- * from and joined back into `stream` (also while `stream` is captured).
+ * An application is a graph launched on `stream`; within it independent blocks of a
+ * stage may run side by side.  With GEMSLR_SOLVE_GRAPH=0 a solve does the same on
+ * streams of the handle, forked from and joined back into `stream`.
  */
 #define GEMSLR_BATCH_RHS 8
 typedef struct gemslr_batch_ctx *gemslr_batch;

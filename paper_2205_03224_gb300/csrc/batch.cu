@@ -1,6 +1,7 @@
 // Batched GeMSLR-FGMRES: many independent systems with up to kBatchRhs
 // right-hand sides each.  Setup (Alg. 1) runs per system; the solve phase
-// launches every stage of M^{-1} (Alg. 2) once over all systems and runs
+// runs every stage of M^{-1} (Alg. 2) over all systems together (one launch, or for a
+// streamed level's substitutions a launch per group of blocks, side by side) and
 // FGMRES (Sec. 4.1) for every (system, rhs) pair in lock step inside one CUDA
 // graph with conditional WHILE nodes.  The preconditioner is FP32 (W in BF16
 // with FP32 accumulation); the Krylov vectors, least-squares problems and
@@ -380,7 +381,7 @@ void build_batch_level(gemslr_batch_ctx *B, int l, bool last, int rows_cta, BLev
     }
 }
 
-// M^{-1} on the batch layout: in (FP64) -> out (FP64), every stage one launch.
+// M^{-1} on the batch layout: in (FP64) -> out (FP64), every stage over all systems.
 // live (nsys flags, or nullptr): systems whose flag is 0 are skipped.
 void batch_apply_layout(gemslr_batch_ctx *B, const double *in, double *out, cudaStream_t st,
                         const int32_t *live = nullptr) {

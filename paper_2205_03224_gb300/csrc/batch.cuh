@@ -1,6 +1,6 @@
 // Device views of a batch of independent GeMSLR systems solved together with
 // kBatchRhs right-hand sides each (the batched workload: many uneven systems,
-// one launch per stage of M^{-1} over all of them).
+// every stage of M^{-1} over all of them).
 //
 // Batch vector layout: the systems one after another, each in its own
 // multilevel order; every row holds kBatchRhs consecutive values (one per

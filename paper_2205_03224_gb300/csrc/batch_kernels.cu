@@ -1,5 +1,5 @@
 // Batched kernels: many independent GeMSLR systems, kBatchRhs right-hand
-// sides each, one launch per stage of M^{-1} (Alg. 2) over every system, and
+// sides each, every stage of M^{-1} (Alg. 2) over all systems together, and
 // FGMRES (Sec. 4.1) run for every (system, rhs) pair in lock step.
 // Preconditioner in FP32 (W in BF16, FP32 accumulation), Krylov in FP64.
 #include <type_traits>

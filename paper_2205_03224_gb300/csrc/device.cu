@@ -649,8 +649,8 @@ void upload_level(const HostLevel &hl, int64_t n, bool schur, Arena &a, DevLevel
     v.S.consumers = sh.consumers;
     // More blocks than SMs: a ring that leaves room for up to three CTAs on an SM, in FP32
     // without the four warps that only help (their registers are another CTA's).  us per
-    // application with a CTA per SM / now: 96^3 in 1,024 blocks mixed 370 / 204, FP64 1315 /
-    // 1146; 64^3 in 256 mixed 142 / 90, FP64 483 / 392, complex 975 / 913.
+    // application with a CTA per SM / now: 96^3 in 1,024 blocks mixed 370 / 210, FP64 1315 /
+    // 1148; 64^3 in 256 mixed 142 / 92, FP64 483 / 392, complex 975 / 911.
     int dev = 0, sms = 1, per_sm = 0;
     GEMSLR_CUDA(cudaGetDevice(&dev));
     GEMSLR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

@@ -1,7 +1,7 @@
 // Device primitives shared by the kernels: warp reductions, deterministic
-// column reductions of per-CTA partial sums, the mbarrier / bulk-copy (TMA,
-// non-tensor) PTX of the staged substitution kernels, and the lane-per-row
-// chunk consumer.
+// column reductions of per-CTA partial sums, and the mbarrier / bulk-copy (TMA,
+// non-tensor) PTX of the staged substitution kernels with the chunk ring of the
+// batched ones.
 #pragma once
 
 #include <cstdint>
@@ -148,9 +148,10 @@ __device__ __forceinline__ bool poll_warp(uint64_t *bar, unsigned parity, volati
     return __all_sync(0xffffffffu, poll_bounded(bar, parity, abort_flag, limit));
 }
 // One bulk copy global -> shared (16-byte aligned addresses, size a multiple of
-// 16).  The factor chunks are read once per application, so the copy marks
-// them evict-first in L2: the vectors that the substitutions gather from (in
-// global memory for blocks too large for shared memory) keep their L2 lines.
+// 16).  A sweep reads its factors once, and only a Schur level's up sweep, after all
+// the levels below, reads the same ones again, so the copy marks them evict-first in
+// L2: the vectors that the substitutions gather from (in global memory for blocks
+// too large for shared memory) keep their L2 lines.
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
     uint64_t policy;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
