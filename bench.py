@@ -51,27 +51,27 @@ FP64_PEAK_GFLOPS = 152 * 2 * 2.07 * 2
 #   M^-1 kernels: (config, precision, kernel) -> DRAM bytes of a launch
 #   Krylov kernels (work grows with the step j): -> (DRAM bytes, algorithmic bytes) of the captured step
 TRAFFIC_SOURCES = ["trsv.cu", "kernels.cu", "kernels.cuh", "stream.cuh", "lowrank.cuh", "ptx.cuh", "device.cu"]
-NCU_TRAFFIC_DIGEST = "916bf152ac449417"
+NCU_TRAFFIC_DIGEST = "a7629b29958003c0"
 NCU_TRAFFIC = {
-    ("c2", "mixed", "trsv_down_L0"): 43_714_560,
-    ("c2", "mixed", "trsv_down_L1"): 6_465_280,
-    ("c2", "mixed", "trsv_down_L2"): 449_536,
-    ("c2", "mixed", "trsv_last"): 158_208,
-    ("c2", "mixed", "trsv_up_L2"): 292_352,
-    ("c2", "mixed", "trsv_up_L1"): 4_825_344,
-    ("c2", "mixed", "trsv_up_L0"): 45_555_200,
-    ("c2", "fp64", "trsv_down_L0"): 73_524_736 + 430_336,
-    ("c2", "fp64", "trsv_down_L1"): 15_524_608,
-    ("c2", "fp64", "trsv_down_L2"): 1_221_376,
-    ("c2", "fp64", "trsv_last"): 341_760,
-    ("c2", "fp64", "trsv_up_L2"): 462_592,
-    ("c2", "fp64", "trsv_up_L1"): 7_983_360,
-    ("c2", "fp64", "trsv_up_L0"): 76_710_400 + 49_408,
+    ("c2", "mixed", "trsv_down_L0"): 42_088_960,
+    ("c2", "mixed", "trsv_down_L1"): 7_454_720,
+    ("c2", "mixed", "trsv_down_L2"): 784_640,
+    ("c2", "mixed", "trsv_last"): 243_968,
+    ("c2", "mixed", "trsv_up_L2"): 625_408,
+    ("c2", "mixed", "trsv_up_L1"): 5_813_504,
+    ("c2", "mixed", "trsv_up_L0"): 43_931_648 + 768,
+    ("c2", "fp64", "trsv_down_L0"): 91_379_200 + 1_959_168,
+    ("c2", "fp64", "trsv_down_L1"): 19_908_864,
+    ("c2", "fp64", "trsv_down_L2"): 1_853_952,
+    ("c2", "fp64", "trsv_last"): 485_632,
+    ("c2", "fp64", "trsv_up_L2"): 1_093_120,
+    ("c2", "fp64", "trsv_up_L1"): 12_372_736,
+    ("c2", "fp64", "trsv_up_L0"): 94_557_184 + 244_480,
 }
 NCU_TRAFFIC_KRYLOV = {
-    ("c2", "mixed", "dgs_fix_adots"): (54_606_080 + 174_080, None),
-    ("c2", "mixed", "dgs_spmv_dots"): (80_565_248 + 2_691_840, None),
-    ("c2", "mixed", "dgs_next"): (56_636_672 + 102_656, None),
+    ("c2", "mixed", "dgs_fix_adots"): (54_612_480 + 52_224, None),
+    ("c2", "mixed", "dgs_spmv_dots"): (80_578_048 + 475_136, None),
+    ("c2", "mixed", "dgs_next"): (56_635_392 + 1_280, None),
 }
 NCU_KRYLOV_STEP = 25
 
