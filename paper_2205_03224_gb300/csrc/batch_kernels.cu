@@ -39,15 +39,15 @@ __device__ __forceinline__ bool last_of(unsigned *counter, unsigned n) {
 // then work[rows] -= result.  Without SMEM (blocks too large even for RPC = 1)
 // RPC is kBatchRhs and the vector stays in global memory.
 // Bound by a row's gathers, one chunk of rows after another: four entries (shared
-// memory) or six (global memory) are in flight at a time, written out because the
+// memory) or ten (global memory) are in flight at a time, written out because the
 // compiler's own choice changes with the code around it, and the next chunk is
 // looked for before the sums.  In global memory the gathers have to hit in L1, so
 // the carve-out leaves it all but two CTAs' rings (set_btrsv_smem_limit): when the
 // kernel takes only 32 registers a third CTA would fit, the driver gives shared
 // memory the whole SM for it, and an application of 8 systems of 56^3 took 4.18 ms
-// instead of 2.68.  Now 2.58; 96 systems (sides 16 to 48), rows of up to 20 entries,
-// 5.50 ms (7.68; with 48 registers and no such figure 5.55); 24 of them (10 to 20), in
-// shared memory, 0.71 (0.72).
+// instead of 2.68.  Now 2.55; 96 systems (sides 16 to 48), rows of up to 20 entries,
+// 5.44 ms (7.68; with 48 registers 5.55); 20 of 50^3 2.85 (six in flight 2.96; 2.91); 24
+// (10 to 20), rows of up to 20, in shared memory, 0.71 (0.72).
 template <int MODE, bool SMEM, int RPC>
 __global__ void __launch_bounds__(kBatchTrsvThreads)
 k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ work, double *__restrict__ out_final,
@@ -154,7 +154,7 @@ k_btrsv(const BatchLevel lv, const double *__restrict__ in, float *__restrict__ 
                     a1 += v[1] * x[1];
                     a0 += v[2] * x[2];
                 } else {
-#pragma unroll 3
+#pragma unroll 5
                     for (; q + 1 < len; q += 2) {
                         a0 += vals[q * nrow + t] * xs[cols[q * nrow + t] * RPC + r];
                         a1 += vals[(q + 1) * nrow + t] * xs[cols[(q + 1) * nrow + t] * RPC + r];
